@@ -30,7 +30,10 @@ __device__ __forceinline__ bool hs_in_bounds(long long idx, long long n) {
 // Operator kinds as compiled into kernels.
 // OP_BOX27: the HPCG 27-point system (diagonal 27, -1 on the 26 neighbours of
 // the 3x3x3 box), applied through separable box sums (3-D only).
-enum OpKind : int { OP_SYM = 0, OP_NONSYM = 1, OP_VARK = 2, OP_BOX27 = 3 };
+// OP_ISO (FP64 only): OP_SYM with one coupling for all neighbours (equal
+// spacings, or HPCG's 7-point matrix), applied through the neighbours' sum,
+// which runs on the integer pipes (hs_fx.cuh).
+enum OpKind : int { OP_SYM = 0, OP_NONSYM = 1, OP_VARK = 2, OP_BOX27 = 3, OP_ISO = 4 };
 
 // Device status word values (mirrors hs_status where they overlap).
 enum DevStatus : int {

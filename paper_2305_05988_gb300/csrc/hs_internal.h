@@ -96,6 +96,16 @@ struct ConstRow {
 };
 ConstRow const_row(const hs_op* A);
 
+// The operator kind a kernel is compiled for: FP64 operators with one coupling
+// for all neighbours take OP_ISO.
+inline int kernel_op(const hs_op* A, hs_dtype dt) {
+  const int opk = opkind_of(A);
+  if (opk != OP_SYM || dt != HS_F64 || A->ndim < 2) return opk;
+  const ConstRow c = const_row(A);
+  const bool iso = c.xl == c.xu && c.yl == c.xu && c.yu == c.xu && (A->ndim < 3 || (c.zl == c.xu && c.zu == c.xu));
+  return iso ? OP_ISO : OP_SYM;
+}
+
 // Chooses a tiling (rows per tile, z chunk length) for `grid` persistent
 // blocks, or for a one-item-per-block launch when grid == 0.
 Tiling choose_tiling(const Geom& g, int by, int grid, bool src_expensive, int planes = 0, int cx = 1);

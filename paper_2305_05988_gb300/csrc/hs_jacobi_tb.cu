@@ -17,7 +17,8 @@
 // bound) and costs FP64 ones the ring recomputation; both are measured.
 //
 // Every node runs the same Jacobi-form arithmetic as k_jacobi (jacobi_apply,
-// same operand order), so the iterates are bitwise those of single sweeps.
+// same operand order, the same neighbour sum for OP_ISO), so the iterates are
+// bitwise those of single sweeps.
 #include <algorithm>
 #include <cmath>
 
@@ -62,7 +63,7 @@ __host__ __device__ constexpr int tb_smem_values() { return S * 2 * tb_w<S>() * 
 // every shared read of step t is of a plane written in step t - 1, so one
 // barrier per step suffices.  The chunk starts S planes early (levels fill
 // up) and runs S planes past its end (level S needs level S - 1 one plane up).
-template <typename T, int S>
+template <typename T, int OPK, int S>
 __device__ void tb_item(const JacTbArgs<T>& a, int item, int L, const T* __restrict__ src, T* __restrict__ dst,
                         T* sm) {
   constexpr int W = tb_w<S>(), H = tb_h<S>(), PL = W * H;
@@ -123,7 +124,11 @@ __device__ void tb_item(const JacTbArgs<T>& a, int item, int L, const T* __restr
         nb.n = pl[c + W];
         nb.b = q[s - 1][0];
         nb.t = q[s - 1][2];
-        v = jacobi_apply<T, OP_SYM, 3>(a.cf, OpRaw<T, OP_SYM>{}, nb, bdq[S - s]);
+        if constexpr (OPK == OP_ISO) {
+          const Fx f[6] = {fx_make(nb.w), fx_make(nb.e), fx_make(nb.s), fx_make(nb.n), fx_make(nb.b), fx_make(nb.t)};
+          nb.box = fx_total(f);
+        }
+        v = jacobi_apply<T, OPK, 3>(a.cf, OpRaw<T, OPK>{}, nb, bdq[S - s]);
         if (s == L && p >= z0 && p < z1 && tx >= S && tx < W - S && ty >= S && ty < H - S)
           dst[(long long)p * P + col] = v;
       }
@@ -141,7 +146,7 @@ __device__ void tb_item(const JacTbArgs<T>& a, int item, int L, const T* __restr
   }
 }
 
-template <typename T, int S>
+template <typename T, int OPK, int S>
 __global__ void __launch_bounds__(tb_threads<S>()) k_jacobi_tb(JacTbArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ double sh[32 * MAX_SCAL];
@@ -165,7 +170,7 @@ __global__ void __launch_bounds__(tb_threads<S>()) k_jacobi_tb(JacTbArgs<T> a) {
   T* dst = a.x1;
   for (int done = 0; done < a.sweeps;) {
     const int L = min(S, a.sweeps - done);
-    for (int item = blockIdx.x; item < a.tl.items(); item += gridDim.x) tb_item<T, S>(a, item, L, src, dst, sm);
+    for (int item = blockIdx.x; item < a.tl.items(); item += gridDim.x) tb_item<T, OPK, S>(a, item, L, src, dst, sm);
     if (!grid_sync(a.cm.ctrl, a.cm.partials, sh)) return;
     done += L;
     T* tmp = const_cast<T*>(src);
@@ -178,7 +183,7 @@ __global__ void __launch_bounds__(tb_threads<S>()) k_jacobi_tb(JacTbArgs<T> a) {
   finish(a.cm.ctrl, DS_CONVERGED, a.sweeps, -1.0);
 }
 
-template <typename T, int S>
+template <typename T, int OPK, int S>
 static hs_status jacobi_tb_t(const SolveArgs& sa, hs_result* res, double* hist) {
   const hs_op* A = sa.A;
   const Geom g = geom_of(A);
@@ -212,8 +217,8 @@ static hs_status jacobi_tb_t(const SolveArgs& sa, hs_result* res, double* hist) 
   const int block = tb_threads<S>();
   const size_t smem = (size_t)tb_smem_values<S>() * sizeof(T);
   int per_sm = 0;
-  cudaError_t e = cudaFuncSetAttribute(k_jacobi_tb<T, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_jacobi_tb<T, S>, block, smem);
+  cudaError_t e = cudaFuncSetAttribute(k_jacobi_tb<T, OPK, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_jacobi_tb<T, OPK, S>, block, smem);
   if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
   if (per_sm < 1) {
     set_error("temporally blocked Jacobi cannot be resident");
@@ -225,7 +230,7 @@ static hs_status jacobi_tb_t(const SolveArgs& sa, hs_result* res, double* hist) 
   grid = std::max(1, std::min(grid, tl.items()));
   a.tl = tl;
   void* args[] = {&a};
-  s = launch_coop((const void*)k_jacobi_tb<T, S>, grid, block, args, smem, sa.stream);
+  s = launch_coop((const void*)k_jacobi_tb<T, OPK, S>, grid, block, args, smem, sa.stream);
   if (s != HS_OK) return s;
   return finish_solve_pub(sa, cm, nullptr, nullptr, nullptr, nullptr, a.x1, res, hist, false);
 }
@@ -236,16 +241,18 @@ bool jacobi_tb_applies(const SolveArgs& sa) {
   return sa.o.sweeps_per_pass >= 2 && sa.tol == 0.0 && sa.A->ndim == 3 && opkind_of(sa.A) == OP_SYM;
 }
 
-hs_status run_jacobi_tb(const SolveArgs& sa, hs_result* res, double* hist) {
+template <typename T, int OPK>
+static hs_status jacobi_tb_s(const SolveArgs& sa, hs_result* res, double* hist) {
   const int S = std::min(sa.o.sweeps_per_pass, 4);
-  if (sa.dtype == HS_F64) {
-    if (S == 2) return jacobi_tb_t<double, 2>(sa, res, hist);
-    if (S == 3) return jacobi_tb_t<double, 3>(sa, res, hist);
-    return jacobi_tb_t<double, 4>(sa, res, hist);
-  }
-  if (S == 2) return jacobi_tb_t<float, 2>(sa, res, hist);
-  if (S == 3) return jacobi_tb_t<float, 3>(sa, res, hist);
-  return jacobi_tb_t<float, 4>(sa, res, hist);
+  if (S == 2) return jacobi_tb_t<T, OPK, 2>(sa, res, hist);
+  if (S == 3) return jacobi_tb_t<T, OPK, 3>(sa, res, hist);
+  return jacobi_tb_t<T, OPK, 4>(sa, res, hist);
+}
+
+hs_status run_jacobi_tb(const SolveArgs& sa, hs_result* res, double* hist) {
+  if (sa.dtype == HS_F32) return jacobi_tb_s<float, OP_SYM>(sa, res, hist);
+  return kernel_op(sa.A, sa.dtype) == OP_ISO ? jacobi_tb_s<double, OP_ISO>(sa, res, hist)
+                                             : jacobi_tb_s<double, OP_SYM>(sa, res, hist);
 }
 
 }  // namespace hs

@@ -136,6 +136,7 @@ struct JacArgs {
 template <typename T, int OPK, int NDIM, bool FUSE>
 struct JacobiSink {
   static constexpr bool kBox = OPK == OP_BOX27;
+  static constexpr bool kIso = OPK == OP_ISO;
   Coef<T> cf;
   Geom g;
   const T* bsrc;   // b/a_ii (constant) or b (variable)
@@ -145,6 +146,9 @@ struct JacobiSink {
     OpRaw<T, OPK> o;
     T b;
   };
+  static constexpr int NB = 1, kAux = 99;
+  __device__ __forceinline__ const T* opnd(int) const { return bsrc; }
+  __device__ __forceinline__ Raw pack(const T (&v)[1], T) const { return Raw{{}, v[0]}; }
   __device__ __forceinline__ Raw fetch(long long idx, int i, int j, int k) const {
     return Raw{op_fetch<T, OPK, NDIM>(cf, g, idx, i, j, k), __ldcg(bsrc + idx)};
   }
@@ -159,8 +163,24 @@ struct JacobiSink {
   }
 };
 
+// Register caps of the neighbour-sum engine's 3-D kernels (A/B at 256^3):
+// Jacobi 64 (107 us per sweep; 48: 125, 56: 111, 80: 110), CG 80 (241 us per
+// iteration; 56: 278, 64: 258, 72: 250, 96: 283), BiCGStab 80 (527; 64: 642,
+// 96: 570, 128: 552).
+#ifndef HS_JAC_ISO_MAXNREG
+#define HS_JAC_ISO_MAXNREG 64
+#endif
+#ifndef HS_CG_ISO_MAXNREG
+#define HS_CG_ISO_MAXNREG 80
+#endif
+#ifndef HS_BI_ISO_MAXNREG
+#define HS_BI_ISO_MAXNREG 80
+#endif
+template <typename T, int OPK, int NDIM>
+constexpr int jac_maxnreg() { return OPK == OP_ISO && NDIM == 3 ? HS_JAC_ISO_MAXNREG : 128; }
+
 template <typename T, int OPK, int NDIM, bool FUSE>
-__global__ void __launch_bounds__(512) k_jacobi(JacArgs<T> a) {
+__global__ void __launch_bounds__(512) __maxnreg__((jac_maxnreg<T, OPK, NDIM>())) k_jacobi(JacArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ double sh[32 * MAX_SCAL];
   T* sm = reinterpret_cast<T*>(smraw);
@@ -257,20 +277,22 @@ __global__ void __launch_bounds__(512) k_jacobi(JacArgs<T> a) {
 #ifndef HS_BI32_MAXNREG
 #define HS_BI32_MAXNREG 64
 #endif
-template <typename T, int OPK>
+template <typename T, int OPK, int NDIM>
 constexpr int cg_maxnreg() {
+  if (OPK == OP_ISO && NDIM == 3) return HS_CG_ISO_MAXNREG;
   if (sizeof(T) == 4) return (HS_CG32_MAXNREG > 0 && OPK == OP_VARK) ? HS_CG32_MAXNREG : 255;
   if (OPK == OP_VARK) return HS_CGV64_MAXNREG > 0 ? HS_CGV64_MAXNREG : 255;
   return HS_CG_MAXNREG > 0 ? HS_CG_MAXNREG : 255;
 }
-template <typename T, int OPK>
+template <typename T, int OPK, int NDIM>
 constexpr int bi_maxnreg() {
+  if (OPK == OP_ISO && NDIM == 3) return HS_BI_ISO_MAXNREG;
   if (sizeof(T) == 4) return HS_BI32_MAXNREG > 0 ? HS_BI32_MAXNREG : 255;
   return HS_BI_MAXNREG > 0 ? HS_BI_MAXNREG : 255;
 }
 
 template <typename T, int OPK, int NDIM>
-__global__ void __launch_bounds__(512) __maxnreg__((cg_maxnreg<T, OPK>())) k_cg(CgArgs<T> a) {
+__global__ void __launch_bounds__(512) __maxnreg__((cg_maxnreg<T, OPK, NDIM>())) k_cg(CgArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ double sh[32 * MAX_SCAL];
   const Team tm = grid_team(a.cm.ctrl, a.cm.partials);
@@ -279,7 +301,7 @@ __global__ void __launch_bounds__(512) __maxnreg__((cg_maxnreg<T, OPK>())) k_cg(
 }
 
 template <typename T, int OPK, int NDIM>
-__global__ void __launch_bounds__(512) __maxnreg__((bi_maxnreg<T, OPK>())) k_bicgstab(BiArgs<T> a) {
+__global__ void __launch_bounds__(512) __maxnreg__((bi_maxnreg<T, OPK, NDIM>())) k_bicgstab(BiArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ double sh[32 * MAX_SCAL];
   const Team tm = grid_team(a.cm.ctrl, a.cm.partials);
@@ -447,6 +469,8 @@ static hs_status dispatch(hs_dtype dt, int opk, int ndim, F&& f) {
   if (dt == HS_F64) {
     HS_CASE(double, OP_SYM, 2)
     HS_CASE(double, OP_SYM, 3)
+    HS_CASE(double, OP_ISO, 2)
+    HS_CASE(double, OP_ISO, 3)
     HS_CASE(double, OP_NONSYM, 2)
     HS_CASE(double, OP_NONSYM, 3)
     HS_CASE(double, OP_VARK, 2)
@@ -525,10 +549,10 @@ static hs_status spmv_vark_direct(const hs_op* A, const void* x, void* y, cudaSt
   double ih[3];
   for (int d = 0; d < 3; d++) ih[d] = d < A->ndim ? 1.0 / (A->h[d] * A->h[d]) : 0.0;
   if (A->kdt == HS_F64)
-    k_spmv_vark_direct<T, double, NDIM><<<tl.items(), 32 * by, slab_bytes<T>(by, CX_ST), st>>>(
+    k_spmv_vark_direct<T, double, NDIM><<<tl.items(), 32 * by, slab_bytes<T, OP_VARK>(by, CX_ST), st>>>(
         g, tl, (const double*)A->k, ih[0], ih[1], ih[2], (const T*)x, (T*)y);
   else
-    k_spmv_vark_direct<T, float, NDIM><<<tl.items(), 32 * by, slab_bytes<T>(by, CX_ST), st>>>(
+    k_spmv_vark_direct<T, float, NDIM><<<tl.items(), 32 * by, slab_bytes<T, OP_VARK>(by, CX_ST), st>>>(
         g, tl, (const float*)A->k, ih[0], ih[1], ih[2], (const T*)x, (T*)y);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? HS_OK : cuda_fail(e, "spmv launch");
@@ -536,7 +560,7 @@ static hs_status spmv_vark_direct(const hs_op* A, const void* x, void* y, cudaSt
 
 hs_status run_spmv(const hs_op* A, hs_dtype dt, const void* x, void* y, cudaStream_t st) {
   Geom g = geom_of(A);
-  return dispatch(dt, opkind_of(A), A->ndim, [&](auto tag) -> hs_status {
+  return dispatch(dt, kernel_op(A, dt), A->ndim, [&](auto tag) -> hs_status {
     using Tg = decltype(tag);
     using T = typename Tg::T;
     constexpr int OPK = Tg::OPK, NDIM = Tg::NDIM;
@@ -545,7 +569,7 @@ hs_status run_spmv(const hs_op* A, hs_dtype dt, const void* x, void* y, cudaStre
     Coef<T> cf = op_coef<T>(A, nullptr, nullptr, nullptr, nullptr, &sigma);
     int by = rows_per_tile(g);
     Tiling tl = choose_tiling(g, by, 0, false, 0, cx_st<OPK>());
-    k_spmv<T, OPK, NDIM><<<tl.items(), 32 * by, slab_bytes<T>(by, cx_st<OPK>()), st>>>(g, tl, cf, (T)sigma, (const T*)x, (T*)y);
+    k_spmv<T, OPK, NDIM><<<tl.items(), 32 * by, slab_bytes<T, OPK>(by, cx_st<OPK>()), st>>>(g, tl, cf, (T)sigma, (const T*)x, (T*)y);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? hs_dbg_take(st) : cuda_fail(e, "spmv launch");
   });
@@ -565,7 +589,7 @@ hs_status run_residual_plain(const hs_op* A, hs_dtype dt, const void* b, const v
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? hs_dbg_take(st) : cuda_fail(e, "residual launch");
   }
-  return dispatch(dt, opkind_of(A), A->ndim, [&](auto tag) -> hs_status {
+  return dispatch(dt, kernel_op(A, dt), A->ndim, [&](auto tag) -> hs_status {
     using Tg = decltype(tag);
     using T = typename Tg::T;
     constexpr int OPK = Tg::OPK, NDIM = Tg::NDIM;
@@ -574,7 +598,7 @@ hs_status run_residual_plain(const hs_op* A, hs_dtype dt, const void* b, const v
     Coef<T> cf = op_coef<T>(A, nullptr, nullptr, nullptr, nullptr, &sigma);
     int by = rows_per_tile(g);
     Tiling tl = choose_tiling(g, by, 0, false, 0, cx_st<OPK>());
-    k_residual<T, OPK, NDIM><<<tl.items(), 32 * by, slab_bytes<T>(by, cx_st<OPK>()), st>>>(g, tl, cf, (T)sigma, (const T*)b,
+    k_residual<T, OPK, NDIM><<<tl.items(), 32 * by, slab_bytes<T, OPK>(by, cx_st<OPK>()), st>>>(g, tl, cf, (T)sigma, (const T*)b,
                                                                                (const T*)x, (T*)r, nullptr);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? hs_dbg_take(st) : cuda_fail(e, "residual launch");
@@ -587,7 +611,7 @@ static hs_status residual_norms(const hs_op* A, hs_dtype dt, const void* D, cons
                                 const void* az, const void* b, const void* x, void* r, double* norms_dev,
                                 double* partials_dev, cudaStream_t st) {
   Geom g = geom_of(A);
-  return dispatch(dt, opkind_of(A), A->ndim, [&](auto tag) -> hs_status {
+  return dispatch(dt, kernel_op(A, dt), A->ndim, [&](auto tag) -> hs_status {
     using Tg = decltype(tag);
     using T = typename Tg::T;
     constexpr int OPK = Tg::OPK, NDIM = Tg::NDIM;
@@ -597,7 +621,7 @@ static hs_status residual_norms(const hs_op* A, hs_dtype dt, const void* D, cons
     constexpr int cx = cx_st<OPK>();   // must match the kernel's columns per lane
     Tiling tl = choose_tiling(g, by, 0, false, 0, cx);
     int grid = std::min(tl.items(), MAX_BLOCKS * MAX_SCAL / 2);
-    k_residual<T, OPK, NDIM><<<grid, 32 * by, slab_bytes<T>(by, cx), st>>>(g, tl, cf, (T)sigma, (const T*)b,
+    k_residual<T, OPK, NDIM><<<grid, 32 * by, slab_bytes<T, OPK>(by, cx), st>>>(g, tl, cf, (T)sigma, (const T*)b,
                                                                         (const T*)x, (T*)r, partials_dev);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "residual launch");
@@ -753,7 +777,7 @@ hs_status finish_solve_pub(const SolveArgs& sa, const Common& cm, const void* D,
 // ---- Jacobi -----------------------------------------------------------------
 hs_status run_jacobi(const SolveArgs& sa, hs_result* res, double* hist) {
   if (jacobi_tb_applies(sa)) return run_jacobi_tb(sa, res, hist);
-  return dispatch(sa.dtype, opkind_of(sa.A), sa.A->ndim, [&](auto tag) -> hs_status {
+  return dispatch(sa.dtype, kernel_op(sa.A, sa.dtype), sa.A->ndim, [&](auto tag) -> hs_status {
     using Tg = decltype(tag);
     using T = typename Tg::T;
     constexpr int OPK = Tg::OPK, NDIM = Tg::NDIM;
@@ -797,7 +821,7 @@ hs_status run_jacobi(const SolveArgs& sa, hs_result* res, double* hist) {
     a.fuse = sa.tol > 0.0 ? 1 : 0;
     int by = rows_for(g, sa.o);
     constexpr int cx = cx_jac<T, OPK>();
-    size_t smem = slab_bytes<T>(by, cx);
+    size_t smem = slab_bytes<T, OPK>(by, cx);
     int grid = 0;
     const void* kern = a.fuse ? (const void*)k_jacobi<T, OPK, NDIM, true> : (const void*)k_jacobi<T, OPK, NDIM, false>;
     s = a.fuse ? plan_persistent(k_jacobi<T, OPK, NDIM, true>, 32 * by, smem, g, by, false, &grid, &a.tl, sa.o, cx)
@@ -836,7 +860,7 @@ static hs_status cg_core(const hs_op* A, const Coef<T>& cf, double sigma, const 
   if (s != HS_OK) return s;
   int by = rows_for(a.g, o);
   constexpr int cx = cx_cg<T, OPK>();
-  size_t smem = slab_bytes<T>(by, cx);
+  size_t smem = slab_bytes<T, OPK>(by, cx, 2, 1);
   int grid = 0;
   s = plan_persistent(k_cg<T, OPK, NDIM>, 32 * by, smem, a.g, by, true, &grid, &a.tl, o, cx);
   if (s != HS_OK) return s;
@@ -871,7 +895,7 @@ static hs_status bicgstab_core(const hs_op* A, const Coef<T>& cf, double sigma, 
   hs_status s = init_ctrl(cm, o, st);
   if (s != HS_OK) return s;
   int by = rows_for(a.g, o);
-  size_t smem = slab_bytes<T>(by, CX_BI);
+  size_t smem = slab_bytes<T, OPK>(by, CX_BI, 3, 1);
   int grid = 0;
   s = plan_persistent(k_bicgstab<T, OPK, NDIM>, 32 * by, smem, a.g, by, true, &grid, &a.tl, o, CX_BI);
   if (s != HS_OK) return s;
@@ -881,7 +905,7 @@ static hs_status bicgstab_core(const hs_op* A, const Coef<T>& cf, double sigma, 
 
 // ---- CG -----------------------------------------------------------------------
 hs_status run_cg(const SolveArgs& sa, hs_result* res, double* hist) {
-  return dispatch(sa.dtype, opkind_of(sa.A), sa.A->ndim, [&](auto tag) -> hs_status {
+  return dispatch(sa.dtype, kernel_op(sa.A, sa.dtype), sa.A->ndim, [&](auto tag) -> hs_status {
     using Tg = decltype(tag);
     using T = typename Tg::T;
     constexpr int OPK = Tg::OPK, NDIM = Tg::NDIM;
@@ -965,7 +989,7 @@ static hs_status copy_bicgstab_trace(const double* trace, int maxit, int iters, 
 }
 
 hs_status run_bicgstab(const SolveArgs& sa, hs_result* res, double* hist) {
-  return dispatch(sa.dtype, opkind_of(sa.A), sa.A->ndim, [&](auto tag) -> hs_status {
+  return dispatch(sa.dtype, kernel_op(sa.A, sa.dtype), sa.A->ndim, [&](auto tag) -> hs_status {
     using Tg = decltype(tag);
     using T = typename Tg::T;
     constexpr int OPK = Tg::OPK, NDIM = Tg::NDIM;

@@ -16,7 +16,7 @@ namespace hs {
 // single-pass SpMV / residual kernels use two.
 constexpr int CX_ST = 2;    // SpMV / residual (7-point operators)
 template <int OPK>
-__host__ __device__ constexpr int cx_st() { return OPK == OP_BOX27 ? 1 : CX_ST; }
+__host__ __device__ constexpr int cx_st() { return OPK == OP_BOX27 || OPK == OP_ISO ? 1 : CX_ST; }
 constexpr int CX_BI = 1;    // BiCGStab
 // FP32 Jacobi: two columns per lane (measured at 256^3: 91 -> 64 us/sweep;
 // the FP32 sweep is memory-latency bound and gains from the second chain).
@@ -84,11 +84,15 @@ __device__ __forceinline__ void team_finish(const Team& tm, const BodyOut& o) {
 template <typename T, int OPK, int NDIM>
 struct SpmvSink {
   static constexpr bool kBox = OPK == OP_BOX27;
+  static constexpr bool kIso = OPK == OP_ISO;
   Coef<T> cf;
   Geom g;
   T sigma;
   T* y;
   using Raw = OpRaw<T, OPK>;
+  static constexpr int NB = 0, kAux = 99;
+  __device__ __forceinline__ const T* opnd(int) const { return nullptr; }
+  __device__ __forceinline__ Raw pack(const T (&)[1], T) const { return Raw{}; }
   __device__ __forceinline__ Raw fetch(long long idx, int i, int j, int k) const {
     return op_fetch<T, OPK, NDIM>(cf, g, idx, i, j, k);
   }
@@ -103,6 +107,7 @@ struct SpmvSink {
 template <typename T, int OPK, int NDIM>
 struct ResidualSink {
   static constexpr bool kBox = OPK == OP_BOX27;
+  static constexpr bool kIso = OPK == OP_ISO;
   Coef<T> cf;
   Geom g;
   T sigma;
@@ -113,6 +118,9 @@ struct ResidualSink {
     OpRaw<T, OPK> o;
     T b;
   };
+  static constexpr int NB = 1, kAux = 99;
+  __device__ __forceinline__ const T* opnd(int) const { return b; }
+  __device__ __forceinline__ Raw pack(const T (&v)[1], T) const { return Raw{{}, v[0]}; }
   __device__ __forceinline__ Raw fetch(long long idx, int i, int j, int k) const {
     return Raw{op_fetch<T, OPK, NDIM>(cf, g, idx, i, j, k), __ldg(b + idx)};
   }
@@ -164,9 +172,12 @@ struct PUpdateSrc {
   T* pnew;
   T beta;
   bool first;
+  static constexpr int NA = 2;
   struct Raw {
     T r, p;
   };
+  __device__ __forceinline__ const T* arr(int a) const { return a == 0 ? r : first ? r : pold; }
+  __device__ __forceinline__ Raw pack(const T (&v)[2]) const { return Raw{v[0], v[1]}; }
   __device__ __forceinline__ Raw fetch(long long idx) const {
     Raw q;
     q.r = __ldcg(r + idx);
@@ -187,6 +198,7 @@ struct PUpdateSrc {
 template <typename T, int OPK, int NDIM, bool XUPD>
 struct ApDotSink {
   static constexpr bool kBox = OPK == OP_BOX27;
+  static constexpr bool kIso = OPK == OP_ISO;
   Coef<T> cf;
   Geom g;
   T* w;
@@ -194,17 +206,27 @@ struct ApDotSink {
   const T* pold;
   T ax;
   double acc[1];
-  using Raw = OpRaw<T, OPK>;
+  struct Raw {
+    OpRaw<T, OPK> o;
+    T x, p;   // OP_ISO with XUPD: staged by the engine
+  };
+  static constexpr int NB = XUPD ? 1 : 0, kAux = XUPD ? 1 : 99;   // p_old is the source's operand 1
+  __device__ __forceinline__ const T* opnd(int) const { return x; }
+  __device__ __forceinline__ Raw pack(const T (&v)[1], T p) const { return Raw{{}, v[0], p}; }
   __device__ __forceinline__ Raw fetch(long long idx, int i, int j, int k) const {
-    return op_fetch<T, OPK, NDIM>(cf, g, idx, i, j, k);
+    return Raw{op_fetch<T, OPK, NDIM>(cf, g, idx, i, j, k), T(0), T(0)};
   }
-  __device__ __forceinline__ void operator()(long long idx, const Nbr<T>& nb, const Raw& o, int, int, int) {
-    T wv = op_apply<T, OPK, NDIM>(cf, o, nb);
+  __device__ __forceinline__ void operator()(long long idx, const Nbr<T>& nb, const Raw& q, int, int, int) {
+    T wv = op_apply<T, OPK, NDIM>(cf, q.o, nb);
     w[idx] = wv;
     acc[0] += widen(nb.c) * widen(wv);
-    // p_old was read two planes earlier by the source: an L2 hit; not
-    // prefetched, which would raise the register count of every pass
-    if constexpr (XUPD) x[idx] = fma(ax, __ldcg(pold + idx), __ldcg(x + idx));
+    if constexpr (XUPD && kIso) {
+      x[idx] = fma(ax, q.p, q.x);
+    } else if constexpr (XUPD) {
+      // p_old was read two planes earlier by the source: an L2 hit; not
+      // prefetched, which would raise the register count of every pass
+      x[idx] = fma(ax, __ldcg(pold + idx), __ldcg(x + idx));
+    }
   }
 };
 
@@ -402,9 +424,15 @@ struct BiPSrc {
   const T* vold;
   T* pnew;
   T beta, ws;
+  static constexpr int NA = RESTART ? 1 : 3;
   struct Raw {
     T r, p, v;
   };
+  __device__ __forceinline__ const T* arr(int a) const { return a == 0 ? r : a == 1 ? pold : vold; }
+  __device__ __forceinline__ Raw pack(const T (&q)[NA]) const {
+    if constexpr (RESTART) return Raw{q[0], T(0), T(0)};
+    else return Raw{q[0], q[1], q[2]};
+  }
   __device__ __forceinline__ Raw fetch(long long idx) const {
     Raw q;
     q.r = __ldcg(r + idx);
@@ -432,6 +460,7 @@ struct BiPSrc {
 template <typename T, int OPK, int NDIM, bool RESTART>
 struct BiVSink {
   static constexpr bool kBox = OPK == OP_BOX27;
+  static constexpr bool kIso = OPK == OP_ISO;
   Coef<T> cf;
   Geom g;
   const T* r;
@@ -443,6 +472,9 @@ struct BiVSink {
     OpRaw<T, OPK> o;
     T q;   // r (restart) or r'
   };
+  static constexpr int NB = 1, kAux = 99;
+  __device__ __forceinline__ const T* opnd(int) const { return RESTART ? r : rs; }
+  __device__ __forceinline__ Raw pack(const T (&v)[1], T) const { return Raw{{}, v[0]}; }
   __device__ __forceinline__ Raw fetch(long long idx, int i, int j, int k) const {
     return Raw{op_fetch<T, OPK, NDIM>(cf, g, idx, i, j, k), RESTART ? __ldcg(r + idx) : __ldcg(rs + idx)};
   }
@@ -465,9 +497,12 @@ struct BiSSrc {
   const T* v;
   T* s;
   T as;
+  static constexpr int NA = 2;
   struct Raw {
     T r, v;
   };
+  __device__ __forceinline__ const T* arr(int a) const { return a == 0 ? r : v; }
+  __device__ __forceinline__ Raw pack(const T (&q)[2]) const { return Raw{q[0], q[1]}; }
   __device__ __forceinline__ Raw fetch(long long idx) const { return Raw{__ldcg(r + idx), __ldcg(v + idx)}; }
   __device__ __forceinline__ T make(const Raw& q, long long idx, bool own) const {
     T sv = fma(-as, q.v, q.r);
@@ -480,11 +515,15 @@ struct BiSSrc {
 template <typename T, int OPK, int NDIM>
 struct BiTSink {
   static constexpr bool kBox = OPK == OP_BOX27;
+  static constexpr bool kIso = OPK == OP_ISO;
   Coef<T> cf;
   Geom g;
   T* t;
   double acc[3];
   using Raw = OpRaw<T, OPK>;
+  static constexpr int NB = 0, kAux = 99;
+  __device__ __forceinline__ const T* opnd(int) const { return nullptr; }
+  __device__ __forceinline__ Raw pack(const T (&)[1], T) const { return Raw{}; }
   __device__ __forceinline__ Raw fetch(long long idx, int i, int j, int k) const {
     return op_fetch<T, OPK, NDIM>(cf, g, idx, i, j, k);
   }
@@ -710,11 +749,6 @@ inline int rows_for(const Geom& g, const hs_opts& o) {
   return rows_per_tile(g);
 }
 
-template <typename T>
-inline size_t slab_bytes(int by, int cx) {
-  return (size_t)2 * (by + 2) * (BX * cx + 2) * sizeof(T);
-}
-
 // Operator coefficients for stencil kernels (scaled form, or var-k arrays).
 template <typename T>
 inline Coef<T> op_coef(const hs_op* A, const void* D, const void* ax, const void* ay, const void* az,
@@ -736,7 +770,10 @@ template <typename K>
 inline hs_status plan_persistent(K kernel, int block, size_t smem, const Geom& g, int by, bool src_expensive,
                                  int* grid_out, Tiling* tl_out, const hs_opts& o, int cx) {
   int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, smem);
+  cudaError_t e = cudaSuccess;
+  if (smem > 48 * 1024)
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, smem);
   if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
   if (per_sm < 1) {
     set_error("persistent kernel cannot be resident (block %d, smem %zu)", block, smem);

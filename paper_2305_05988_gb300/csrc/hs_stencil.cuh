@@ -18,10 +18,15 @@
 #include <type_traits>
 
 #include "hs_common.cuh"
+#include "hs_fx.cuh"
 
 namespace hs {
 
 constexpr int BX = 32;
+#ifndef HS_FX_NS
+#define HS_FX_NS 4
+#endif
+constexpr int FX_NS = HS_FX_NS;   // ring stages of the neighbour-sum engine
 
 struct Tiling {
   int by;        // rows per tile (3..16), blockDim.x = 32 * by
@@ -45,6 +50,15 @@ __device__ __forceinline__ void decode_item(const Tiling& t, const Geom& g, int 
   z1 = min(g.nz, z0 + t.lz);
 }
 
+// Bytes of shared memory of the engine for
+// `by` rows; na, nb: staged operands of the source and the sink (OP_ISO).
+template <typename T, int OPK>
+inline size_t slab_bytes(int by, int cx, int na = 1, int nb = 1) {
+  const size_t pl = (size_t)(by + 2) * (BX * cx + 2);
+  if (OPK != OP_ISO) return 2 * pl * sizeof(T);
+  return 24 * pl + 8 * (size_t)FX_NS * (na * (32 * by + 96) + nb * 32 * by);
+}
+
 // Shared slab: 2 planes of (by + 2) x (32 CX + 2) values.
 template <typename T, int CX>
 __device__ __forceinline__ T& slab(T* sm, int by, int buf, int row, int col) {
@@ -52,7 +66,8 @@ __device__ __forceinline__ T& slab(T* sm, int by, int buf, int row, int col) {
 }
 
 // Neighbour values of the current node handed to the stencil functor (box:
-// the sum over the node's 3x3x3 box, center included, for OP_BOX27 sinks).
+// the sum over the node's 3x3x3 box, center included, for OP_BOX27 sinks; the
+// sum of the node's neighbours for OP_ISO sinks).
 template <typename T>
 struct Nbr {
   T c, w, e, s, n, b, t;
@@ -65,6 +80,13 @@ template <class S, class = void>
 struct is_box_sink : std::false_type {};
 template <class S>
 struct is_box_sink<S, std::void_t<decltype(S::kBox)>> : std::integral_constant<bool, S::kBox> {};
+
+// A sink that takes the neighbours' sum declares kIso = true; the tile engine
+// then stages integer significands and hands it the sum in Nbr::box.
+template <class S, class = void>
+struct is_iso_sink : std::false_type {};
+template <class S>
+struct is_iso_sink<S, std::void_t<decltype(S::kIso)>> : std::integral_constant<bool, S::kIso> {};
 
 // Process one work item, software-pipelined along z.
 //
@@ -87,12 +109,21 @@ template <typename T, class Src, class Sink>
 __device__ __forceinline__ void zmarch_box(const Geom& g, const Tiling& tl, int item, T* sm, const Src& src,
                                            Sink& sink);
 
+template <int NDIM, class Src, class Sink>
+__device__ __forceinline__ void zmarch_iso(const Geom& g, const Tiling& tl, int item, double* sm, const Src& src,
+                                           Sink& sink);
+
 template <typename T, int NDIM, int CX, class Src, class Sink>
 __device__ __forceinline__ void zmarch_item(const Geom& g, const Tiling& tl, int item, T* sm, const Src& src,
                                             Sink& sink) {
   if constexpr (is_box_sink<Sink>::value) {
     static_assert(NDIM == 3 && CX == 1, "the 27-point engine is 3-D with one column per lane");
     zmarch_box<T>(g, tl, item, sm, src, sink);
+    return;
+  }
+  if constexpr (is_iso_sink<Sink>::value) {
+    static_assert(std::is_same<T, double>::value && CX == 1, "the neighbour-sum engine is FP64, one column per lane");
+    zmarch_iso<NDIM>(g, tl, item, sm, src, sink);
     return;
   }
   using SR = typename Src::Raw;
@@ -369,16 +400,225 @@ __device__ __forceinline__ void zmarch_box(const Geom& g, const Tiling& tl, int 
   __syncthreads();   // the next item restages the shared plane
 }
 
+// The neighbour-sum engine (OP_ISO): work items of zmarch_item, one column per
+// lane.  Every value the source produces is split into significand and
+// exponent once (fx_make); the slab and the column registers hold the split
+// form, and the sink receives c and the sum of its neighbours.
+//
+// With the additions off the FP64 pipe the march is bound by instruction issue
+// and by how many loads are in flight, so operands are staged by cp.async in a
+// ring of NS steps private to each thread: group k holds the source's
+// operands of plane k + 1 (own column and halo node) and the sink's of plane
+// k.  No register waits on memory, columns and planes outside the grid are
+// zero-filled by the copy, and no load needs a branch.  The copies go through
+// L1; a value rewritten by another block was ordered by the grid barrier's
+// acquire, which also drops stale L1 lines.
+//
+// 256^3 FP64, before (zmarch_item, additions on the FP64 pipe) and now: Jacobi
+// 220 -> 114 us per sweep (59 us of traffic), CG 411 -> 245 us per iteration,
+// SpMV 256 -> 122 us, residual 327 -> 181 us.  Tried and slower: operands
+// prefetched in registers as in zmarch_item (Jacobi 135, CG 289), one plane
+// ahead only (Jacobi 173), the loop unrolled six times so that no register
+// moves (CG 366: the code leaves the instruction cache), two rows per lane
+// (Jacobi 149).
+//
+// Shared memory: two slab buffers of (by + 2) x 34 significands (8 bytes) and
+// exponents (4 bytes), then NS ring stages of NA (32 by + 96) + NB 32 by
+// doubles.
+__device__ __forceinline__ void cp_async8(unsigned dst, const double* src, unsigned bytes) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int n>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(n) : "memory");
+}
+__device__ __forceinline__ double ld_shared(unsigned a) {
+  double v;
+  asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+  return v;
+}
+
+template <int NDIM, class Src, class Sink>
+__device__ __forceinline__ void zmarch_iso(const Geom& g, const Tiling& tl, int item, double* sm, const Src& src,
+                                           Sink& sink) {
+  constexpr int SW = BX + 2, NA = Src::NA, NB = Sink::NB;
+  int i0, j0, z0, z1;
+  decode_item(tl, g, item, i0, j0, z0, z1);
+  const int by = tl.by;
+  const int pl = (by + 2) * SW;
+  const int lx = threadIdx.x & 31, ly = threadIdx.x >> 5;
+  const int i = i0 + lx, j = j0 + ly;
+  const bool inside = (i < g.nx) && (j < g.ny);
+  const unsigned P = (unsigned)g.plane;
+  const int c0 = (ly + 1) * SW + lx + 1;
+  // the halo node of this thread (one at most)
+  int hc = -1, hi = 0, hj = 0;
+  if (ly == 0) {
+    hi = i; hj = j0 - 1; hc = lx + 1;
+  } else if (ly == 1) {
+    hi = i; hj = j0 + by; hc = (by + 1) * SW + lx + 1;
+  } else if (ly == 2) {
+    if (lx < by) {
+      hi = i0 - 1; hj = j0 + lx; hc = (lx + 1) * SW;
+    } else if (lx >= 16 && lx < 16 + by) {
+      hi = i0 + BX; hj = j0 + lx - 16; hc = (lx - 15) * SW + BX + 1;
+    }
+  }
+  const bool hin = hc >= 0 && hi >= 0 && hi < g.nx && hj >= 0 && hj < g.ny;
+  // element indices at plane 0 of the columns (N < 2^31); 0 outside the grid
+  const unsigned oc = inside ? (unsigned)j * (unsigned)g.nx + (unsigned)i : 0u;
+  const unsigned hcol = hin ? (unsigned)hj * (unsigned)g.nx + (unsigned)hi : 0u;
+  const unsigned in8 = inside ? 8u : 0u, hin8 = hin ? 8u : 0u;
+
+  const unsigned sm0 = (unsigned)__cvta_generic_to_shared(sm);
+  const unsigned nthr = 32u * (unsigned)by;
+  const unsigned stage = 8u * (NA * (nthr + 96u) + NB * nthr);
+  const unsigned ring0 = sm0 + 24u * (unsigned)pl + 8u * threadIdx.x;
+  const unsigned hoff = 8u * NA * nthr;                  // halo slots
+  const unsigned koff = hoff + 8u * NA * 96u;            // sink slots
+  // group of step k: source plane k + 1 (planes up to min(z1, nz - 1), halo up
+  // to z1 - 1), sink plane k; past those the copies fill in zeros
+  auto issue = [&](int k) {
+    const unsigned at = ring0 + (unsigned)((k - z0) & (FX_NS - 1)) * stage;
+    const unsigned up = (unsigned)min(k + 1, g.nz - 1) * P;
+    const unsigned sz = k + 1 <= z1 && k + 1 < g.nz ? in8 : 0u;
+#pragma unroll
+    for (int a = 0; a < NA; a++)
+      if (HS_IN_BOUNDS(oc + up, g.N)) cp_async8(at + 8u * a * nthr, src.arr(a) + (oc + up), sz);
+    if (hc >= 0) {
+      const unsigned hsz = k + 1 < z1 ? hin8 : 0u;
+#pragma unroll
+      for (int a = 0; a < NA; a++)
+        if (HS_IN_BOUNDS(hcol + up, g.N)) cp_async8(at + hoff + 8u * a * 96u, src.arr(a) + (hcol + up), hsz);
+    }
+    if (NB > 0) {
+      const unsigned here = (unsigned)min(k, g.nz - 1) * P;
+      const unsigned ksz = k < z1 ? in8 : 0u;
+#pragma unroll
+      for (int b = 0; b < NB; b++)
+        if (HS_IN_BOUNDS(oc + here, g.N)) cp_async8(at + koff + 8u * b * nthr, sink.opnd(b) + (oc + here), ksz);
+    }
+    cp_async_commit();
+  };
+  // slab addresses of this thread's node and halo node in buffer 0
+  const unsigned sigc = sm0 + 8u * (unsigned)c0, expc = sm0 + 8u * (unsigned)pl + 4u * (unsigned)c0;
+  const unsigned sigh = sm0 + 8u * (unsigned)hc, exph = sm0 + 8u * (unsigned)pl + 4u * (unsigned)hc;
+  auto put = [&](unsigned sig, unsigned ex, const Fx& f) {
+    asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(sig), "r"(f.lo), "r"(f.hi) : "memory");
+    asm volatile("st.shared.b32 [%0], %1;" ::"r"(ex), "r"(f.e) : "memory");
+  };
+  auto get = [&](unsigned sig, unsigned ex) -> Fx {
+    Fx f;
+    asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(f.lo), "=r"(f.hi) : "r"(sig) : "memory");
+    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(f.e) : "r"(ex) : "memory");
+    return f;
+  };
+
+  if (NDIM == 3) {
+#pragma unroll
+    for (int n = 0; n < FX_NS - 1; n++) issue(z0 + n);
+  }
+  // planes z0 - 1 and z0 straight from memory
+  Fx fb = {0u, 0, 0u}, fc = fb;
+  double vc = 0.0, aux = 0.0, ko[NB > 0 ? NB : 1];
+  unsigned o = oc + (unsigned)z0 * P;
+  if (inside && HS_IN_BOUNDS(o, g.N)) {
+    double ra[NA], rc[NA];
+    const bool low = NDIM == 3 && z0 > 0;
+#pragma unroll
+    for (int a = 0; a < NA; a++) {
+      ra[a] = low ? __ldcg(src.arr(a) + (o - P)) : 0.0;
+      rc[a] = __ldcg(src.arr(a) + o);
+    }
+    if (low) fb = fx_make(src.make(src.pack(ra), o - P, false));
+    if (NDIM == 2) {
+#pragma unroll
+      for (int b = 0; b < NB; b++) ko[b] = __ldcg(sink.opnd(b) + o);
+    }
+    vc = src.make(src.pack(rc), o, true);
+    fc = fx_make(vc);
+    aux = rc[Sink::kAux < NA ? Sink::kAux : 0];
+  }
+  put(sigc, expc, fc);
+  if (hc >= 0) {
+    Fx fh = {0u, 0, 0u};
+    if (hin) {
+      double rh[NA];
+#pragma unroll
+      for (int a = 0; a < NA; a++) rh[a] = __ldcg(src.arr(a) + (hcol + (unsigned)z0 * P));
+      fh = fx_make(src.make(src.pack(rh), hcol + (unsigned)z0 * P, false));
+    }
+    put(sigh, exph, fh);
+  }
+  __syncthreads();
+
+  if constexpr (NDIM == 2) {
+    if (inside) {
+      Nbr<double> nb;
+      nb.c = vc;
+      nb.w = nb.e = nb.s = nb.n = nb.b = nb.t = 0.0;
+      const Fx f[4] = {get(sigc - 8u, expc - 4u), get(sigc + 8u, expc + 4u), get(sigc - 8u * SW, expc - 4u * SW),
+                       get(sigc + 8u * SW, expc + 4u * SW)};
+      nb.box = fx_total(f);
+      if (HS_IN_BOUNDS(o, g.N)) sink(o, nb, sink.pack(ko, aux), i, j, 0);
+    }
+    __syncthreads();
+  } else {
+#pragma unroll 1
+    for (int k = z0; k < z1; k++) {
+      issue(k + FX_NS - 1);
+      cp_async_wait<FX_NS - 1>();
+      const unsigned use = ring0 + (unsigned)((k - z0) & (FX_NS - 1)) * stage;
+      const unsigned cur = (unsigned)((k - z0) & 1) * 12u * (unsigned)pl, next = 12u * (unsigned)pl - cur;
+      double rt[NA];
+#pragma unroll
+      for (int a = 0; a < NA; a++) rt[a] = ld_shared(use + 8u * a * nthr);
+      const double vt = src.make(src.pack(rt), o + P, k + 1 < z1 && inside);
+      const Fx ft = fx_make(vt);
+      put(sigc + next, expc + next, ft);
+      if (hc >= 0) {
+        double rh[NA];
+#pragma unroll
+        for (int a = 0; a < NA; a++) rh[a] = ld_shared(use + hoff + 8u * a * 96u);
+        put(sigh + next, exph + next, fx_make(src.make(src.pack(rh), 0, false)));
+      }
+      if (inside) {
+#pragma unroll
+        for (int b = 0; b < NB; b++) ko[b] = ld_shared(use + koff + 8u * b * nthr);
+        const unsigned sg = sigc + cur, eg = expc + cur;
+        Nbr<double> nb;
+        nb.c = vc;
+        nb.w = nb.e = nb.s = nb.n = nb.b = nb.t = 0.0;
+        const Fx f[6] = {get(sg - 8u, eg - 4u), get(sg + 8u, eg + 4u), get(sg - 8u * SW, eg - 4u * SW),
+                         get(sg + 8u * SW, eg + 4u * SW), fb, ft};
+        nb.box = fx_total(f);
+        if (HS_IN_BOUNDS(o, g.N)) sink(o, nb, sink.pack(ko, aux), i, j, k);
+      }
+      o += P;
+      fb = fc;
+      fc = ft;
+      vc = vt;
+      if (Sink::kAux < NA) aux = rt[Sink::kAux < NA ? Sink::kAux : 0];
+      __syncthreads();
+    }
+    cp_async_wait<0>();   // the next item refills the ring
+  }
+}
+
 // Plain load of one vector as the stencil input.  CG = true reads through
 // L2 only (data written earlier in the same persistent kernel).
 template <typename T, bool CG>
 struct LoadSrc {
+  static constexpr int NA = 1;
   const T* x;
   struct Raw {
     T v;
   };
   __device__ __forceinline__ Raw fetch(long long idx) const { return Raw{CG ? __ldcg(x + idx) : __ldg(x + idx)}; }
   __device__ __forceinline__ T make(const Raw& r, long long, bool) const { return r.v; }
+  __device__ __forceinline__ const T* arr(int) const { return x; }
+  __device__ __forceinline__ Raw pack(const T (&v)[1]) const { return Raw{v[0]}; }
 };
 
 // ---------------------------------------------------------------------------
@@ -427,6 +667,8 @@ __device__ __forceinline__ T op_apply(const Coef<T>& cf, const OpRaw<T, OPK>& o,
   if constexpr (OPK == OP_BOX27) {
     // 27 c - (box - c), with cf.d = 28: 1 instruction after the box sums
     return fma(cf.d, nb.c, -nb.box);
+  } else if constexpr (OPK == OP_ISO) {
+    return fma(cf.d, nb.c, -nb.box);
   } else if constexpr (OPK == OP_SYM) {
     T y = fma(cf.d, nb.c, -(nb.w + nb.e));
     y = fma(cf.yl, nb.s + nb.n, y);
@@ -465,6 +707,8 @@ __device__ __forceinline__ T jacobi_apply(const Coef<T>& cf, const OpRaw<T, OPK>
   if constexpr (OPK == OP_BOX27) {
     // b/a_ii + (box - c)/27: the 26 neighbours all couple with -1
     return fma(cf.xl, nb.box - nb.c, bv);
+  } else if constexpr (OPK == OP_ISO) {
+    return fma(cf.xl, nb.box, bv);
   } else if constexpr (OPK == OP_SYM) {
     T y = fma(cf.xl, nb.w + nb.e, bv);
     y = fma(cf.yl, nb.s + nb.n, y);
