@@ -30,10 +30,12 @@ __device__ __forceinline__ bool hs_in_bounds(long long idx, long long n) {
 // Operator kinds as compiled into kernels.
 // OP_BOX27: the HPCG 27-point system (diagonal 27, -1 on the 26 neighbours of
 // the 3x3x3 box), applied through separable box sums (3-D only).
-// OP_ISO (FP64 only): OP_SYM with one coupling for all neighbours (equal
-// spacings, or HPCG's 7-point matrix), applied through the neighbours' sum,
-// which runs on the integer pipes (hs_fx.cuh).
-enum OpKind : int { OP_SYM = 0, OP_NONSYM = 1, OP_VARK = 2, OP_BOX27 = 3, OP_ISO = 4 };
+// FP64 only, applied through a neighbour sum on the integer pipes (hs_fx.cuh):
+// OP_ISO, an OP_SYM operator with one coupling for all neighbours (equal
+// spacings, or HPCG's 7-point matrix); OP_WSYM and OP_WNON, OP_SYM and
+// OP_NONSYM operators whose couplings lie within a factor of 64.
+enum OpKind : int { OP_SYM = 0, OP_NONSYM = 1, OP_VARK = 2, OP_BOX27 = 3, OP_ISO = 4, OP_WSYM = 5, OP_WNON = 6 };
+__host__ __device__ constexpr bool fx_op(int opk) { return opk >= OP_ISO; }
 
 // Device status word values (mirrors hs_status where they overlap).
 enum DevStatus : int {
@@ -53,8 +55,27 @@ enum DevStatus : int {
 // couplings ax/ay/az (positive), the upper faces taken from the neighbour's
 // lower face:  y_i = D_i c - ax_i W - ax_{i+1} E - ay_i S - ay_{i+nx} N
 //                         - az_i B - az_{i+nx ny} T.
+//
+// FxW: the couplings of an OP_WSYM / OP_WNON operator relative to the upper x
+// one, in the order xl, xu, yl, yu, zl, zu: as doubles w, and as fixed-point
+// fractions of 2^k, c = w 2^(62 - k) < 2^61 in limbs of 31 bits (ch, cl);
+// rc = the rounding constant of a product (see fx_scale).
+struct FxW {
+  double w[6];
+  int ch[6], cl[6];
+  unsigned rc[6];
+  int k;
+};
+
 template <typename T>
-struct Coef {
+struct CoefFx {};
+template <>
+struct CoefFx<double> {
+  FxW fx;
+};
+
+template <typename T>
+struct Coef : CoefFx<T> {
   T d, xl, xu, yl, yu, zl, zu;
   const T* D;
   const T* ax;

@@ -11,13 +11,16 @@
 //
 // Accuracy: a term loses less than 2^-59 of the largest term's power of two
 // when it is shifted, so n <= 7 terms are summed to within 7 x 2^-59 of it
-// before the one rounding; a chain of FP64 additions rounds n - 1 times at
+// before the one rounding (weighted sums: 6 x 2^-57 of the largest weighted
+// one); a chain of FP64 additions rounds n - 1 times at
 // 2^-53 of its partial sums.  Sums that cancel below 2^-16 of the largest
-// term, terms outside 2^-943 .. 2^1016 and non-finite terms take the FP64
+// term, terms outside 2^-943 .. 2^1006 and non-finite terms take the FP64
 // additions themselves (fx_value restores every double exactly, zeros,
 // subnormals, infinities and NaNs included).
 #pragma once
 #include <cuda_runtime.h>
+
+#include "hs_common.cuh"
 
 namespace hs {
 
@@ -53,41 +56,98 @@ __device__ __forceinline__ double fx_value(const Fx& f) {
                           (int)__funnelshift_r(lo, hi, 7));
 }
 
+// Rounds acc 2^(top - 1023 - 59) to binary64; false (y untouched) where the
+// sum has cancelled or the exponents leave the range this path handles.
+__device__ __forceinline__ bool fx_round(long long acc, unsigned top, double& y) {
+  const int s = (int)(acc >> 63);
+  const unsigned long long a = (unsigned long long)((acc ^ (long long)s) - (long long)s);
+  const unsigned ah = (unsigned)(a >> 32), al = (unsigned)a;
+  if (!(top - 80u < 1950u && ah >= 0x1000u)) return false;
+  int z;                                                       // leading zeros of ah: 1 .. 19
+  asm("bfind.shiftamt.u32 %0, %1;" : "=r"(z) : "r"(ah));
+  z -= 1;
+  // leading bit to 2^62, round to nearest even at 2^10 (a tie is one sum in
+  // eight or four when the exponents are close: rounded away from zero it
+  // would bias the sums by 2^-57, which a solve's smooth error accumulates)
+  const unsigned tl = al << z;
+  const unsigned long long t =
+      (((unsigned long long)__funnelshift_l(al, ah, z) << 32) | tl) + (511u + ((tl >> 10) & 1u));
+  const unsigned lo = (unsigned)(t >> 10);
+  const unsigned hi = (unsigned)(t >> 42) + ((top + 2u) << 20) - ((unsigned)z << 20);
+  y = __hiloint2double((int)(hi | ((unsigned)s & 0x80000000u)), (int)lo);
+  return true;
+}
+
+// The significand shifted to the exponent top >= f.e.
+__device__ __forceinline__ long long fx_align(const Fx& f, unsigned top) {
+  long long m = ((long long)f.hi << 32) | f.lo;
+  asm("shr.s64 %0, %0, %1;" : "+l"(m) : "r"(top - f.e));   // amounts above 63 leave the sign
+  return m;
+}
+
+template <int n>
+__device__ __forceinline__ unsigned fx_top(const Fx (&v)[n]) {
+  unsigned top = v[0].e;
+#pragma unroll
+  for (int q = 1; q < n; q++) top = max(top, v[q].e);
+  return top;
+}
+
 // v[0] + ... + v[n-1]
 template <int n>
 __device__ __forceinline__ double fx_total(const Fx (&v)[n]) {
   static_assert(n >= 2 && n <= 7, "three bits of headroom above 2^60");
-  unsigned top = v[0].e;
-#pragma unroll
-  for (int q = 1; q < n; q++) top = max(top, v[q].e);
+  const unsigned top = fx_top(v);
   long long acc = 0;
 #pragma unroll
-  for (int q = 0; q < n; q++) {
-    long long m = ((long long)v[q].hi << 32) | v[q].lo;
-    asm("shr.s64 %0, %0, %1;" : "+l"(m) : "r"(top - v[q].e));   // amounts above 63 leave the sign
-    acc += m;
-  }
-  const int s = (int)(acc >> 63);
-  const unsigned long long a = (unsigned long long)((acc ^ (long long)s) - (long long)s);
-  const unsigned ah = (unsigned)(a >> 32), al = (unsigned)a;
-  if (top - 80u < 1960u && ah >= 0x1000u) {
-    int z;                                                       // leading zeros of ah: 1 .. 19
-    asm("bfind.shiftamt.u32 %0, %1;" : "=r"(z) : "r"(ah));
-    z -= 1;
-    // leading bit to 2^62, round to nearest even at 2^10 (a tie is one sum in
-    // eight or four when the exponents are close: rounded away from zero it
-    // would bias the sums by 2^-57, which a solve's smooth error accumulates)
-    const unsigned tl = al << z;
-    const unsigned long long t =
-        (((unsigned long long)__funnelshift_l(al, ah, z) << 32) | tl) + (511u + ((tl >> 10) & 1u));
-    const unsigned lo = (unsigned)(t >> 10);
-    const unsigned hi = (unsigned)(t >> 42) + ((top + 2u) << 20) - ((unsigned)z << 20);
-    return __hiloint2double((int)(hi | ((unsigned)s & 0x80000000u)), (int)lo);
-  }
-  double y = fx_value(v[0]);
+  for (int q = 0; q < n; q++) acc += fx_align(v[q], top);
+  double y;
+  if (fx_round(acc, top, y)) return y;
+  y = fx_value(v[0]);
 #pragma unroll
   for (int q = 1; q < n; q++) y += fx_value(v[q]);
   return y;
+}
+
+// m c / 2^63 rounded to nearest, |m| < 2^61, c = ch 2^31 + cl < 2^61 (every
+// partial sum below 2^63):
+//   (mh 2^32 + ml)(ch 2^31 + cl) / 2^63 = mh ch + (2 mh cl + ml ch + ml cl / 2^31) / 2^32,
+// the last term replaced by its mean cl (ml is uniform): rc = 2^31 + cl.
+__device__ __forceinline__ long long fx_scale(long long m, const FxW& W, int q) {
+  const int mh = (int)(m >> 32);
+  const unsigned ml = (unsigned)m;
+  long long t, r;
+  asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(t) : "r"(ml), "r"(W.ch[q]), "l"((long long)W.rc[q]));
+  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(t) : "r"(mh + mh), "r"(W.cl[q]));
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(mh), "r"(W.ch[q]), "l"(t >> 32));
+  return r;
+}
+
+// The sum of a node's neighbours in the order w, e, s, n, b, t, weighted by
+// the couplings relative to the upper x one (OP_WSYM, OP_WNON).  Terms are
+// aligned first (exact for exponents up to 7 apart), then scaled with
+// rounding to 2^-57 of the largest coupling's term.
+template <int OPK, int n>
+__device__ __forceinline__ double fx_neighbours(const Fx (&v)[n], const FxW& W) {
+  if constexpr (OPK == OP_ISO) {
+    return fx_total(v);
+  } else {
+    const unsigned top = fx_top(v);
+    long long acc = 0;
+    if constexpr (OPK == OP_WSYM) {
+#pragma unroll
+      for (int q = 0; q < n; q += 2) acc += fx_scale(fx_align(v[q], top) + fx_align(v[q + 1], top), W, q);
+    } else {
+#pragma unroll
+      for (int q = 0; q < n; q++) acc += fx_scale(fx_align(v[q], top), W, q);
+    }
+    double y;
+    if (fx_round(acc, top, y)) return __hiloint2double(__double2hiint(y) + ((W.k + 1) << 20), __double2loint(y));
+    y = W.w[0] * fx_value(v[0]);
+#pragma unroll
+    for (int q = 1; q < n; q++) y = fma(W.w[q], fx_value(v[q]), y);
+    return y;
+  }
 }
 
 }  // namespace hs

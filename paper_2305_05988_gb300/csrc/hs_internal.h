@@ -96,14 +96,24 @@ struct ConstRow {
 };
 ConstRow const_row(const hs_op* A);
 
-// The operator kind a kernel is compiled for: FP64 operators with one coupling
-// for all neighbours take OP_ISO.
+// Fills W with an operator's couplings relative to the upper x one; false if
+// they lie more than a factor of 64 apart.
+bool fx_weights(const hs_op* A, FxW* W);
+
+// The operator kind a kernel is compiled for.  FP64 operators in 2-D and 3-D
+// take the neighbour sum on the integer pipes where the couplings lie within
+// a factor of 64 (grid spacings within 8, cell Peclet numbers to 31): beyond,
+// the fixed-point products would be coarser than FP64's rounding for the
+// weakest coupling.
 inline int kernel_op(const hs_op* A, hs_dtype dt) {
   const int opk = opkind_of(A);
-  if (opk != OP_SYM || dt != HS_F64 || A->ndim < 2) return opk;
-  const ConstRow c = const_row(A);
-  const bool iso = c.xl == c.xu && c.yl == c.xu && c.yu == c.xu && (A->ndim < 3 || (c.zl == c.xu && c.zu == c.xu));
-  return iso ? OP_ISO : OP_SYM;
+  if ((opk != OP_SYM && opk != OP_NONSYM) || dt != HS_F64 || A->ndim < 2) return opk;
+  FxW W;
+  if (!fx_weights(A, &W)) return opk;
+  if (opk == OP_NONSYM) return OP_WNON;
+  for (int q = 0; q < 2 * A->ndim; q++)
+    if (W.w[q] != 1.0) return OP_WSYM;
+  return OP_ISO;
 }
 
 // Chooses a tiling (rows per tile, z chunk length) for `grid` persistent

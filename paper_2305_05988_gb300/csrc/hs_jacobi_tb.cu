@@ -17,7 +17,7 @@
 // bound) and costs FP64 ones the ring recomputation; both are measured.
 //
 // Every node runs the same Jacobi-form arithmetic as k_jacobi (jacobi_apply,
-// same operand order, the same neighbour sum for OP_ISO), so the iterates are
+// same operand order, the same neighbour sum), so the iterates are
 // bitwise those of single sweeps.
 #include <algorithm>
 #include <cmath>
@@ -124,9 +124,9 @@ __device__ void tb_item(const JacTbArgs<T>& a, int item, int L, const T* __restr
         nb.n = pl[c + W];
         nb.b = q[s - 1][0];
         nb.t = q[s - 1][2];
-        if constexpr (OPK == OP_ISO) {
+        if constexpr (fx_op(OPK)) {
           const Fx f[6] = {fx_make(nb.w), fx_make(nb.e), fx_make(nb.s), fx_make(nb.n), fx_make(nb.b), fx_make(nb.t)};
-          nb.box = fx_total(f);
+          nb.box = fx_neighbours<OPK>(f, a.cf.fx);
         }
         v = jacobi_apply<T, OPK, 3>(a.cf, OpRaw<T, OPK>{}, nb, bdq[S - s]);
         if (s == L && p >= z0 && p < z1 && tx >= S && tx < W - S && ty >= S && ty < H - S)
@@ -207,6 +207,7 @@ static hs_status jacobi_tb_t(const SolveArgs& sa, hs_result* res, double* hist) 
     a.cf.zl = (T)(-r.zl / r.d);
     a.cf.zu = (T)(-r.zu / r.d);
     a.invd = (T)(1.0 / r.d);
+    if constexpr (std::is_same<T, double>::value) fx_weights(A, &a.cf.fx);
   }
   a.g = g;
   a.b = (const T*)sa.b;
@@ -251,8 +252,10 @@ static hs_status jacobi_tb_s(const SolveArgs& sa, hs_result* res, double* hist) 
 
 hs_status run_jacobi_tb(const SolveArgs& sa, hs_result* res, double* hist) {
   if (sa.dtype == HS_F32) return jacobi_tb_s<float, OP_SYM>(sa, res, hist);
-  return kernel_op(sa.A, sa.dtype) == OP_ISO ? jacobi_tb_s<double, OP_ISO>(sa, res, hist)
-                                             : jacobi_tb_s<double, OP_SYM>(sa, res, hist);
+  const int opk = kernel_op(sa.A, sa.dtype);
+  if (opk == OP_ISO) return jacobi_tb_s<double, OP_ISO>(sa, res, hist);
+  if (opk == OP_WSYM) return jacobi_tb_s<double, OP_WSYM>(sa, res, hist);
+  return jacobi_tb_s<double, OP_SYM>(sa, res, hist);
 }
 
 }  // namespace hs

@@ -136,7 +136,7 @@ struct JacArgs {
 template <typename T, int OPK, int NDIM, bool FUSE>
 struct JacobiSink {
   static constexpr bool kBox = OPK == OP_BOX27;
-  static constexpr bool kIso = OPK == OP_ISO;
+  static constexpr int kOp = OPK;
   Coef<T> cf;
   Geom g;
   const T* bsrc;   // b/a_ii (constant) or b (variable)
@@ -177,7 +177,7 @@ struct JacobiSink {
 #define HS_BI_ISO_MAXNREG 80
 #endif
 template <typename T, int OPK, int NDIM>
-constexpr int jac_maxnreg() { return OPK == OP_ISO && NDIM == 3 ? HS_JAC_ISO_MAXNREG : 128; }
+constexpr int jac_maxnreg() { return fx_op(OPK) && NDIM == 3 ? HS_JAC_ISO_MAXNREG : 128; }
 
 template <typename T, int OPK, int NDIM, bool FUSE>
 __global__ void __launch_bounds__(512) __maxnreg__((jac_maxnreg<T, OPK, NDIM>())) k_jacobi(JacArgs<T> a) {
@@ -279,14 +279,14 @@ __global__ void __launch_bounds__(512) __maxnreg__((jac_maxnreg<T, OPK, NDIM>())
 #endif
 template <typename T, int OPK, int NDIM>
 constexpr int cg_maxnreg() {
-  if (OPK == OP_ISO && NDIM == 3) return HS_CG_ISO_MAXNREG;
+  if (fx_op(OPK) && NDIM == 3) return HS_CG_ISO_MAXNREG;
   if (sizeof(T) == 4) return (HS_CG32_MAXNREG > 0 && OPK == OP_VARK) ? HS_CG32_MAXNREG : 255;
   if (OPK == OP_VARK) return HS_CGV64_MAXNREG > 0 ? HS_CGV64_MAXNREG : 255;
   return HS_CG_MAXNREG > 0 ? HS_CG_MAXNREG : 255;
 }
 template <typename T, int OPK, int NDIM>
 constexpr int bi_maxnreg() {
-  if (OPK == OP_ISO && NDIM == 3) return HS_BI_ISO_MAXNREG;
+  if (fx_op(OPK) && NDIM == 3) return HS_BI_ISO_MAXNREG;
   if (sizeof(T) == 4) return HS_BI32_MAXNREG > 0 ? HS_BI32_MAXNREG : 255;
   return HS_BI_MAXNREG > 0 ? HS_BI_MAXNREG : 255;
 }
@@ -399,6 +399,30 @@ ConstRow const_row(const hs_op* A) {
   return c;
 }
 
+bool fx_weights(const hs_op* A, FxW* W) {
+  const ConstRow c = const_row(A);
+  const double a[6] = {c.xl, c.xu, c.yl, c.yu, c.zl, c.zu};
+  double lo = 1e300, hi = 0.0;
+  *W = FxW{};
+  for (int q = 0; q < 2 * A->ndim; q++) {
+    W->w[q] = a[q] / c.xu;
+    lo = std::min(lo, W->w[q]);
+    hi = std::max(hi, W->w[q]);
+  }
+  if (!(hi <= 64.0 * lo)) return false;
+  // 2^k > 2 max w, so that c = w 2^(62 - k) < 2^61; within a factor of 64 every
+  // c is exact
+  std::frexp(hi, &W->k);
+  W->k += 1;
+  for (int q = 0; q < 2 * A->ndim; q++) {
+    const long long v = (long long)std::ldexp(W->w[q], 62 - W->k);
+    W->ch[q] = (int)(v >> 31);
+    W->cl[q] = (int)(v & 0x7fffffff);
+    W->rc[q] = 0x80000000u + (unsigned)W->cl[q];
+  }
+  return true;
+}
+
 // Jacobi coefficients g = -a/a_ii.
 template <typename T>
 static Coef<T> jacobi_coef(const hs_op* A, T* invd, double* d2) {
@@ -413,6 +437,7 @@ static Coef<T> jacobi_coef(const hs_op* A, T* invd, double* d2) {
   cf.zu = (T)(-c.zu / c.d);
   *invd = (T)(1.0 / c.d);
   *d2 = c.d * c.d;
+  if constexpr (std::is_same<T, double>::value) fx_weights(A, &cf.fx);
   return cf;
 }
 
@@ -471,6 +496,10 @@ static hs_status dispatch(hs_dtype dt, int opk, int ndim, F&& f) {
     HS_CASE(double, OP_SYM, 3)
     HS_CASE(double, OP_ISO, 2)
     HS_CASE(double, OP_ISO, 3)
+    HS_CASE(double, OP_WSYM, 2)
+    HS_CASE(double, OP_WSYM, 3)
+    HS_CASE(double, OP_WNON, 2)
+    HS_CASE(double, OP_WNON, 3)
     HS_CASE(double, OP_NONSYM, 2)
     HS_CASE(double, OP_NONSYM, 3)
     HS_CASE(double, OP_VARK, 2)

@@ -5,6 +5,8 @@
 #pragma once
 #include <math.h>
 
+#include <type_traits>
+
 #include "hs_internal.h"
 
 namespace hs {
@@ -16,7 +18,7 @@ namespace hs {
 // single-pass SpMV / residual kernels use two.
 constexpr int CX_ST = 2;    // SpMV / residual (7-point operators)
 template <int OPK>
-__host__ __device__ constexpr int cx_st() { return OPK == OP_BOX27 || OPK == OP_ISO ? 1 : CX_ST; }
+__host__ __device__ constexpr int cx_st() { return OPK == OP_BOX27 || fx_op(OPK) ? 1 : CX_ST; }
 constexpr int CX_BI = 1;    // BiCGStab
 // FP32 Jacobi: two columns per lane (measured at 256^3: 91 -> 64 us/sweep;
 // the FP32 sweep is memory-latency bound and gains from the second chain).
@@ -84,7 +86,7 @@ __device__ __forceinline__ void team_finish(const Team& tm, const BodyOut& o) {
 template <typename T, int OPK, int NDIM>
 struct SpmvSink {
   static constexpr bool kBox = OPK == OP_BOX27;
-  static constexpr bool kIso = OPK == OP_ISO;
+  static constexpr int kOp = OPK;
   Coef<T> cf;
   Geom g;
   T sigma;
@@ -107,7 +109,7 @@ struct SpmvSink {
 template <typename T, int OPK, int NDIM>
 struct ResidualSink {
   static constexpr bool kBox = OPK == OP_BOX27;
-  static constexpr bool kIso = OPK == OP_ISO;
+  static constexpr int kOp = OPK;
   Coef<T> cf;
   Geom g;
   T sigma;
@@ -198,7 +200,7 @@ struct PUpdateSrc {
 template <typename T, int OPK, int NDIM, bool XUPD>
 struct ApDotSink {
   static constexpr bool kBox = OPK == OP_BOX27;
-  static constexpr bool kIso = OPK == OP_ISO;
+  static constexpr int kOp = OPK;
   Coef<T> cf;
   Geom g;
   T* w;
@@ -208,7 +210,7 @@ struct ApDotSink {
   double acc[1];
   struct Raw {
     OpRaw<T, OPK> o;
-    T x, p;   // OP_ISO with XUPD: staged by the engine
+    T x, p;   // fx_op with XUPD: staged by the engine
   };
   static constexpr int NB = XUPD ? 1 : 0, kAux = XUPD ? 1 : 99;   // p_old is the source's operand 1
   __device__ __forceinline__ const T* opnd(int) const { return x; }
@@ -220,7 +222,7 @@ struct ApDotSink {
     T wv = op_apply<T, OPK, NDIM>(cf, q.o, nb);
     w[idx] = wv;
     acc[0] += widen(nb.c) * widen(wv);
-    if constexpr (XUPD && kIso) {
+    if constexpr (XUPD && fx_op(OPK)) {
       x[idx] = fma(ax, q.p, q.x);
     } else if constexpr (XUPD) {
       // p_old was read two planes earlier by the source: an L2 hit; not
@@ -460,7 +462,7 @@ struct BiPSrc {
 template <typename T, int OPK, int NDIM, bool RESTART>
 struct BiVSink {
   static constexpr bool kBox = OPK == OP_BOX27;
-  static constexpr bool kIso = OPK == OP_ISO;
+  static constexpr int kOp = OPK;
   Coef<T> cf;
   Geom g;
   const T* r;
@@ -515,7 +517,7 @@ struct BiSSrc {
 template <typename T, int OPK, int NDIM>
 struct BiTSink {
   static constexpr bool kBox = OPK == OP_BOX27;
-  static constexpr bool kIso = OPK == OP_ISO;
+  static constexpr int kOp = OPK;
   Coef<T> cf;
   Geom g;
   T* t;
@@ -733,6 +735,7 @@ inline Coef<T> scaled_coef(const hs_op* A, double* sigma) {
   cf.zu = (T)(c.zu / s);
   // 27-point: A x = 27 x - (box - x) = 28 x - box (s = 1)
   if (A->kind == KIND_HPCG27) cf.d = (T)(c.d + 1.0);
+  if constexpr (std::is_same<T, double>::value) fx_weights(A, &cf.fx);
   return cf;
 }
 

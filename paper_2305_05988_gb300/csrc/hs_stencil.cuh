@@ -51,11 +51,11 @@ __device__ __forceinline__ void decode_item(const Tiling& t, const Geom& g, int 
 }
 
 // Bytes of shared memory of the engine for
-// `by` rows; na, nb: staged operands of the source and the sink (OP_ISO).
+// `by` rows; na, nb: staged operands of the source and the sink (fx_op).
 template <typename T, int OPK>
 inline size_t slab_bytes(int by, int cx, int na = 1, int nb = 1) {
   const size_t pl = (size_t)(by + 2) * (BX * cx + 2);
-  if (OPK != OP_ISO) return 2 * pl * sizeof(T);
+  if (!fx_op(OPK)) return 2 * pl * sizeof(T);
   return 24 * pl + 8 * (size_t)FX_NS * (na * (32 * by + 96) + nb * 32 * by);
 }
 
@@ -67,7 +67,7 @@ __device__ __forceinline__ T& slab(T* sm, int by, int buf, int row, int col) {
 
 // Neighbour values of the current node handed to the stencil functor (box:
 // the sum over the node's 3x3x3 box, center included, for OP_BOX27 sinks; the
-// sum of the node's neighbours for OP_ISO sinks).
+// weighted sum of the node's neighbours where fx_op(OPK)).
 template <typename T>
 struct Nbr {
   T c, w, e, s, n, b, t;
@@ -81,12 +81,13 @@ struct is_box_sink : std::false_type {};
 template <class S>
 struct is_box_sink<S, std::void_t<decltype(S::kBox)>> : std::integral_constant<bool, S::kBox> {};
 
-// A sink that takes the neighbours' sum declares kIso = true; the tile engine
-// then stages integer significands and hands it the sum in Nbr::box.
+// A sink of an operator applied through its neighbour sum declares kOp = OPK;
+// the tile engine then stages integer significands and hands it the (weighted)
+// sum in Nbr::box.
 template <class S, class = void>
-struct is_iso_sink : std::false_type {};
+struct is_fx_sink : std::false_type {};
 template <class S>
-struct is_iso_sink<S, std::void_t<decltype(S::kIso)>> : std::integral_constant<bool, S::kIso> {};
+struct is_fx_sink<S, std::void_t<decltype(S::kOp)>> : std::integral_constant<bool, fx_op(S::kOp)> {};
 
 // Process one work item, software-pipelined along z.
 //
@@ -110,7 +111,7 @@ __device__ __forceinline__ void zmarch_box(const Geom& g, const Tiling& tl, int 
                                            Sink& sink);
 
 template <int NDIM, class Src, class Sink>
-__device__ __forceinline__ void zmarch_iso(const Geom& g, const Tiling& tl, int item, double* sm, const Src& src,
+__device__ __forceinline__ void zmarch_fx(const Geom& g, const Tiling& tl, int item, double* sm, const Src& src,
                                            Sink& sink);
 
 template <typename T, int NDIM, int CX, class Src, class Sink>
@@ -121,9 +122,9 @@ __device__ __forceinline__ void zmarch_item(const Geom& g, const Tiling& tl, int
     zmarch_box<T>(g, tl, item, sm, src, sink);
     return;
   }
-  if constexpr (is_iso_sink<Sink>::value) {
+  if constexpr (is_fx_sink<Sink>::value) {
     static_assert(std::is_same<T, double>::value && CX == 1, "the neighbour-sum engine is FP64, one column per lane");
-    zmarch_iso<NDIM>(g, tl, item, sm, src, sink);
+    zmarch_fx<NDIM>(g, tl, item, sm, src, sink);
     return;
   }
   using SR = typename Src::Raw;
@@ -400,7 +401,7 @@ __device__ __forceinline__ void zmarch_box(const Geom& g, const Tiling& tl, int 
   __syncthreads();   // the next item restages the shared plane
 }
 
-// The neighbour-sum engine (OP_ISO): work items of zmarch_item, one column per
+// The neighbour-sum engine (fx_op operators): work items of zmarch_item, one column per
 // lane.  Every value the source produces is split into significand and
 // exponent once (fx_make); the slab and the column registers hold the split
 // form, and the sink receives c and the sum of its neighbours.
@@ -416,7 +417,9 @@ __device__ __forceinline__ void zmarch_box(const Geom& g, const Tiling& tl, int 
 //
 // 256^3 FP64, before (zmarch_item, additions on the FP64 pipe) and now: Jacobi
 // 220 -> 114 us per sweep (59 us of traffic), CG 411 -> 245 us per iteration,
-// SpMV 256 -> 122 us, residual 327 -> 181 us.  Tried and slower: operands
+// SpMV 256 -> 122 us, residual 327 -> 181 us; weighted (250 x 187 x 141):
+// Jacobi 99 -> 64, CG 191 -> 129, BiCGStab 392 -> 284; upwind at 256^3: Jacobi
+// 221 -> 167, BiCGStab 858 -> 603.  Tried and slower: operands
 // prefetched in registers as in zmarch_item (Jacobi 135, CG 289), one plane
 // ahead only (Jacobi 173), the loop unrolled six times so that no register
 // moves (CG 366: the code leaves the instruction cache), two rows per lane
@@ -440,7 +443,7 @@ __device__ __forceinline__ double ld_shared(unsigned a) {
 }
 
 template <int NDIM, class Src, class Sink>
-__device__ __forceinline__ void zmarch_iso(const Geom& g, const Tiling& tl, int item, double* sm, const Src& src,
+__device__ __forceinline__ void zmarch_fx(const Geom& g, const Tiling& tl, int item, double* sm, const Src& src,
                                            Sink& sink) {
   constexpr int SW = BX + 2, NA = Src::NA, NB = Sink::NB;
   int i0, j0, z0, z1;
@@ -560,7 +563,7 @@ __device__ __forceinline__ void zmarch_iso(const Geom& g, const Tiling& tl, int 
       nb.w = nb.e = nb.s = nb.n = nb.b = nb.t = 0.0;
       const Fx f[4] = {get(sigc - 8u, expc - 4u), get(sigc + 8u, expc + 4u), get(sigc - 8u * SW, expc - 4u * SW),
                        get(sigc + 8u * SW, expc + 4u * SW)};
-      nb.box = fx_total(f);
+      nb.box = fx_neighbours<Sink::kOp>(f, sink.cf.fx);
       if (HS_IN_BOUNDS(o, g.N)) sink(o, nb, sink.pack(ko, aux), i, j, 0);
     }
     __syncthreads();
@@ -592,7 +595,7 @@ __device__ __forceinline__ void zmarch_iso(const Geom& g, const Tiling& tl, int 
         nb.w = nb.e = nb.s = nb.n = nb.b = nb.t = 0.0;
         const Fx f[6] = {get(sg - 8u, eg - 4u), get(sg + 8u, eg + 4u), get(sg - 8u * SW, eg - 4u * SW),
                          get(sg + 8u * SW, eg + 4u * SW), fb, ft};
-        nb.box = fx_total(f);
+        nb.box = fx_neighbours<Sink::kOp>(f, sink.cf.fx);
         if (HS_IN_BOUNDS(o, g.N)) sink(o, nb, sink.pack(ko, aux), i, j, k);
       }
       o += P;
@@ -667,7 +670,7 @@ __device__ __forceinline__ T op_apply(const Coef<T>& cf, const OpRaw<T, OPK>& o,
   if constexpr (OPK == OP_BOX27) {
     // 27 c - (box - c), with cf.d = 28: 1 instruction after the box sums
     return fma(cf.d, nb.c, -nb.box);
-  } else if constexpr (OPK == OP_ISO) {
+  } else if constexpr (fx_op(OPK)) {
     return fma(cf.d, nb.c, -nb.box);
   } else if constexpr (OPK == OP_SYM) {
     T y = fma(cf.d, nb.c, -(nb.w + nb.e));
@@ -707,8 +710,8 @@ __device__ __forceinline__ T jacobi_apply(const Coef<T>& cf, const OpRaw<T, OPK>
   if constexpr (OPK == OP_BOX27) {
     // b/a_ii + (box - c)/27: the 26 neighbours all couple with -1
     return fma(cf.xl, nb.box - nb.c, bv);
-  } else if constexpr (OPK == OP_ISO) {
-    return fma(cf.xl, nb.box, bv);
+  } else if constexpr (fx_op(OPK)) {
+    return fma(cf.xu, nb.box, bv);
   } else if constexpr (OPK == OP_SYM) {
     T y = fma(cf.xl, nb.w + nb.e, bv);
     y = fma(cf.yl, nb.s + nb.n, y);
