@@ -100,13 +100,13 @@ struct Geom {
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ double widen(double d) { return d; }
 __device__ __forceinline__ double widen(float f) {
-  const unsigned u = __float_as_uint(f);
-  const unsigned ef = (u >> 23) & 0xffu;
-  const unsigned de = (ef == 0u) ? 0u : (ef == 255u ? 2047u : ef + 896u);
-  const unsigned m = (ef == 0u) ? 0u : (u & 0x7fffffu);
-  const unsigned hi = (u & 0x80000000u) | (de << 20) | (m >> 3);
-  const unsigned lo = (m & 7u) << 29;
-  return __hiloint2double((int)hi, (int)lo);
+  const unsigned u = __float_as_uint(f), a = u & 0x7fffffffu;
+  unsigned hi = (a >> 3) + 0x38000000u;
+  if (a >= 0x7f800000u) hi += 0x38000000u;   // infinity, NaN
+  const bool none = a < 0x00800000u;         // zero, subnormal
+  hi = none ? 0u : hi;
+  const unsigned lo = none ? 0u : u << 29;
+  return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)lo);
 }
 
 // ---------------------------------------------------------------------------

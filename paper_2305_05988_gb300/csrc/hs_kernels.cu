@@ -146,20 +146,24 @@ struct JacobiSink {
     OpRaw<T, OPK> o;
     T b;
   };
-  static constexpr int NB = 1, kAux = 99;
+  static constexpr int NB = 1, kAux = 99, NQ = 1;
   __device__ __forceinline__ const T* opnd(int) const { return bsrc; }
   __device__ __forceinline__ Raw pack(const T (&v)[1], T) const { return Raw{{}, v[0]}; }
+  __device__ __forceinline__ T* out() const { return xd; }
+  __device__ __forceinline__ T value(const Nbr<T>& nb, const OpRaw<T, OPK>& o, T bv) {
+    const T xn = jacobi_apply<T, OPK, NDIM>(cf, o, nb, bv);
+    if constexpr (FUSE) {
+      T d = xn - nb.c;
+      if constexpr (OPK == OP_VARK) d = d / o.d;
+      acc[0] += widen(d) * widen(d);
+    }
+    return xn;
+  }
   __device__ __forceinline__ Raw fetch(long long idx, int i, int j, int k) const {
     return Raw{op_fetch<T, OPK, NDIM>(cf, g, idx, i, j, k), __ldcg(bsrc + idx)};
   }
   __device__ __forceinline__ void operator()(long long idx, const Nbr<T>& nb, const Raw& q, int, int, int) {
-    T xn = jacobi_apply<T, OPK, NDIM>(cf, q.o, nb, q.b);
-    xd[idx] = xn;
-    if constexpr (FUSE) {
-      T d = xn - nb.c;
-      if constexpr (OPK == OP_VARK) d = d / q.o.d;
-      acc[0] += widen(d) * widen(d);
-    }
+    xd[idx] = value(nb, q.o, q.b);
   }
 };
 
@@ -170,17 +174,29 @@ struct JacobiSink {
 #ifndef HS_JAC_ISO_MAXNREG
 #define HS_JAC_ISO_MAXNREG 64
 #endif
+// FP32 engine with four nodes per lane: CG's ring leaves room for two blocks
+// per SM on stored coefficients (128 registers; 80 spill and run at the same
+// 169-171 us per iteration), Jacobi's for three (80).
+#ifndef HS_JACQ_MAXNREG
+#define HS_JACQ_MAXNREG 80
+#endif
+#ifndef HS_CGQ_MAXNREG
+#define HS_CGQ_MAXNREG 128
+#endif
 #ifndef HS_CG_ISO_MAXNREG
 #define HS_CG_ISO_MAXNREG 80
 #endif
 #ifndef HS_BI_ISO_MAXNREG
 #define HS_BI_ISO_MAXNREG 80
 #endif
-template <typename T, int OPK, int NDIM>
-constexpr int jac_maxnreg() { return fx_op(OPK) && NDIM == 3 ? HS_JAC_ISO_MAXNREG : 128; }
+template <typename T, int OPK, int NDIM, int CX>
+constexpr int jac_maxnreg() {
+  if (CX == CX_QUAD) return HS_JACQ_MAXNREG;
+  return fx_op(OPK) && NDIM == 3 ? HS_JAC_ISO_MAXNREG : 128;
+}
 
-template <typename T, int OPK, int NDIM, bool FUSE>
-__global__ void __launch_bounds__(512) __maxnreg__((jac_maxnreg<T, OPK, NDIM>())) k_jacobi(JacArgs<T> a) {
+template <typename T, int OPK, int NDIM, bool FUSE, int CX>
+__global__ void __launch_bounds__(512) __maxnreg__((jac_maxnreg<T, OPK, NDIM, CX>())) k_jacobi(JacArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ double sh[32 * MAX_SCAL];
   T* sm = reinterpret_cast<T*>(smraw);
@@ -213,7 +229,7 @@ __global__ void __launch_bounds__(512) __maxnreg__((jac_maxnreg<T, OPK, NDIM>())
     LoadSrc<T, true> src{xs};
     JacobiSink<T, OPK, NDIM, FUSE> sink{a.cf, a.g, bsrc, xd, {0.0}};
     for (int pos = blockIdx.x; pos < a.tl.items(); pos += gridDim.x)
-      zmarch_item<T, NDIM, (cx_jac<T, OPK>())>(a.g, a.tl, pos, sm, src, sink);
+      zmarch_item<T, NDIM, CX>(a.g, a.tl, pos, sm, src, sink);
     if constexpr (FUSE) {
       block_sum<1>(sink.acc, sh);
       double rr[1];
@@ -277,8 +293,9 @@ __global__ void __launch_bounds__(512) __maxnreg__((jac_maxnreg<T, OPK, NDIM>())
 #ifndef HS_BI32_MAXNREG
 #define HS_BI32_MAXNREG 64
 #endif
-template <typename T, int OPK, int NDIM>
+template <typename T, int OPK, int NDIM, int CX>
 constexpr int cg_maxnreg() {
+  if (CX == CX_QUAD) return HS_CGQ_MAXNREG;
   if (fx_op(OPK) && NDIM == 3) return HS_CG_ISO_MAXNREG;
   if (sizeof(T) == 4) return (HS_CG32_MAXNREG > 0 && OPK == OP_VARK) ? HS_CG32_MAXNREG : 255;
   if (OPK == OP_VARK) return HS_CGV64_MAXNREG > 0 ? HS_CGV64_MAXNREG : 255;
@@ -291,13 +308,13 @@ constexpr int bi_maxnreg() {
   return HS_BI_MAXNREG > 0 ? HS_BI_MAXNREG : 255;
 }
 
-template <typename T, int OPK, int NDIM>
-__global__ void __launch_bounds__(512) __maxnreg__((cg_maxnreg<T, OPK, NDIM>())) k_cg(CgArgs<T> a) {
+template <typename T, int OPK, int NDIM, int CX>
+__global__ void __launch_bounds__(512) __maxnreg__((cg_maxnreg<T, OPK, NDIM, CX>())) k_cg(CgArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ double sh[32 * MAX_SCAL];
   const Team tm = grid_team(a.cm.ctrl, a.cm.partials);
   constexpr bool xdefer = HS_CG_XDEFER && sizeof(T) == 8 && OPK != OP_VARK;
-  team_finish(tm, cg_body<T, OPK, NDIM, cx_cg<T, OPK>(), xdefer>(a, tm, reinterpret_cast<T*>(smraw), sh));
+  team_finish(tm, cg_body<T, OPK, NDIM, CX, xdefer>(a, tm, reinterpret_cast<T*>(smraw), sh));
 }
 
 template <typename T, int OPK, int NDIM>
@@ -848,16 +865,29 @@ hs_status run_jacobi(const SolveArgs& sa, hs_result* res, double* hist) {
     a.maxit = sa.maxit;
     a.tol = sa.tol;
     a.fuse = sa.tol > 0.0 ? 1 : 0;
-    int by = rows_for(g, sa.o);
-    constexpr int cx = cx_jac<T, OPK>();
-    size_t smem = slab_bytes<T, OPK>(by, cx);
-    int grid = 0;
-    const void* kern = a.fuse ? (const void*)k_jacobi<T, OPK, NDIM, true> : (const void*)k_jacobi<T, OPK, NDIM, false>;
-    s = a.fuse ? plan_persistent(k_jacobi<T, OPK, NDIM, true>, 32 * by, smem, g, by, false, &grid, &a.tl, sa.o, cx)
-               : plan_persistent(k_jacobi<T, OPK, NDIM, false>, 32 * by, smem, g, by, false, &grid, &a.tl, sa.o, cx);
-    if (s != HS_OK) return s;
-    void* args[] = {&a};
-    s = launch_coop(kern, grid, 32 * by, args, smem, sa.stream);
+    auto launch = [&](auto kern, int threads, int by, int cx, size_t smem) -> hs_status {
+      int grid = 0;
+      hs_status e = plan_persistent(kern, threads, smem, g, by, false, &grid, &a.tl, sa.o, cx);
+      if (e != HS_OK) return e;
+      void* args[] = {&a};
+      return launch_coop((const void*)kern, grid, threads, args, smem, sa.stream);
+    };
+    bool quad = false;
+    if constexpr (std::is_same<T, float>::value && NDIM == 3 && OPK != OP_BOX27) {
+      if (quad_applies(g, sa.o)) {
+        quad = true;
+        constexpr size_t smem = quad_bytes<LoadSrc<T, true>, JacobiSink<T, OPK, NDIM, false>>();
+        s = a.fuse ? launch(k_jacobi<T, OPK, NDIM, true, CX_QUAD>, 256, QR, QTW / BX, smem)
+                   : launch(k_jacobi<T, OPK, NDIM, false, CX_QUAD>, 256, QR, QTW / BX, smem);
+      }
+    }
+    if (!quad) {
+      const int by = rows_for(g, sa.o);
+      constexpr int cx = cx_jac<T, OPK>();
+      const size_t smem = slab_bytes<T, OPK>(by, cx);
+      s = a.fuse ? launch(k_jacobi<T, OPK, NDIM, true, cx>, 32 * by, by, cx, smem)
+                 : launch(k_jacobi<T, OPK, NDIM, false, cx>, 32 * by, by, cx, smem);
+    }
     if (s != HS_OK) return s;
     if (OPK == OP_VARK && sa.o.true_residual) {
       s = setup_vark(A, sa.dtype, D, ax, ay, az, false, sa.stream);  // un-inverted diagonal
@@ -887,14 +917,23 @@ static hs_status cg_core(const hs_op* A, const Coef<T>& cf, double sigma, const 
   a.tol = tol;
   hs_status s = init_ctrl(cm, o, st);
   if (s != HS_OK) return s;
-  int by = rows_for(a.g, o);
+  auto launch = [&](auto kern, int threads, int by, int cx, size_t smem) -> hs_status {
+    int grid = 0;
+    hs_status e = plan_persistent(kern, threads, smem, a.g, by, true, &grid, &a.tl, o, cx);
+    if (e != HS_OK) return e;
+    void* args[] = {&a};
+    return launch_coop((const void*)kern, grid, threads, args, smem, st);
+  };
+  if constexpr (std::is_same<T, float>::value && NDIM == 3 && OPK != OP_BOX27) {
+    if (quad_applies(a.g, o)) {
+      constexpr size_t smem = std::max(quad_bytes<LoadSrc<T, true>, ResidualSink<T, OPK, NDIM>>(),
+                                       quad_bytes<PUpdateSrc<T>, ApDotSink<T, OPK, NDIM, false>>());
+      return launch(k_cg<T, OPK, NDIM, CX_QUAD>, 256, QR, QTW / BX, smem);
+    }
+  }
+  const int by = rows_for(a.g, o);
   constexpr int cx = cx_cg<T, OPK>();
-  size_t smem = slab_bytes<T, OPK>(by, cx, 2, 1);
-  int grid = 0;
-  s = plan_persistent(k_cg<T, OPK, NDIM>, 32 * by, smem, a.g, by, true, &grid, &a.tl, o, cx);
-  if (s != HS_OK) return s;
-  void* args[] = {&a};
-  return launch_coop((const void*)k_cg<T, OPK, NDIM>, grid, 32 * by, args, smem, st);
+  return launch(k_cg<T, OPK, NDIM, cx>, 32 * by, by, cx, slab_bytes<T, OPK>(by, cx, 2, 1));
 }
 
 template <typename T, int OPK, int NDIM>

@@ -8,6 +8,7 @@
 #include <type_traits>
 
 #include "hs_internal.h"
+#include "hs_quad.cuh"
 
 namespace hs {
 
@@ -120,18 +121,22 @@ struct ResidualSink {
     OpRaw<T, OPK> o;
     T b;
   };
-  static constexpr int NB = 1, kAux = 99;
+  static constexpr int NB = 1, kAux = 99, NQ = 1;
   __device__ __forceinline__ const T* opnd(int) const { return b; }
   __device__ __forceinline__ Raw pack(const T (&v)[1], T) const { return Raw{{}, v[0]}; }
+  __device__ __forceinline__ T* out() const { return r; }
+  __device__ __forceinline__ T value(const Nbr<T>& nb, const OpRaw<T, OPK>& o, T bv) {
+    const T v = op_apply<T, OPK, NDIM>(cf, o, nb);
+    const T rv = (OPK == OP_VARK) ? bv - v : fma(-sigma, v, bv);
+    acc[0] += widen(rv) * widen(rv);
+    acc[1] += widen(bv) * widen(bv);
+    return rv;
+  }
   __device__ __forceinline__ Raw fetch(long long idx, int i, int j, int k) const {
     return Raw{op_fetch<T, OPK, NDIM>(cf, g, idx, i, j, k), __ldg(b + idx)};
   }
   __device__ __forceinline__ void operator()(long long idx, const Nbr<T>& nb, const Raw& q, int, int, int) {
-    T v = op_apply<T, OPK, NDIM>(cf, q.o, nb);
-    T rv = (OPK == OP_VARK) ? q.b - v : fma(-sigma, v, q.b);
-    r[idx] = rv;
-    acc[0] += widen(rv) * widen(rv);
-    acc[1] += widen(q.b) * widen(q.b);
+    r[idx] = value(nb, q.o, q.b);
   }
 };
 
@@ -180,6 +185,9 @@ struct PUpdateSrc {
   };
   __device__ __forceinline__ const T* arr(int a) const { return a == 0 ? r : first ? r : pold; }
   __device__ __forceinline__ Raw pack(const T (&v)[2]) const { return Raw{v[0], v[1]}; }
+  __device__ __forceinline__ void put4(long long idx, const float4& v) const {
+    *reinterpret_cast<float4*>(pnew + idx) = v;
+  }
   __device__ __forceinline__ Raw fetch(long long idx) const {
     Raw q;
     q.r = __ldcg(r + idx);
@@ -218,10 +226,15 @@ struct ApDotSink {
   __device__ __forceinline__ Raw fetch(long long idx, int i, int j, int k) const {
     return Raw{op_fetch<T, OPK, NDIM>(cf, g, idx, i, j, k), T(0), T(0)};
   }
-  __device__ __forceinline__ void operator()(long long idx, const Nbr<T>& nb, const Raw& q, int, int, int) {
-    T wv = op_apply<T, OPK, NDIM>(cf, q.o, nb);
-    w[idx] = wv;
+  static constexpr int NQ = 0;
+  __device__ __forceinline__ T* out() const { return w; }
+  __device__ __forceinline__ T value(const Nbr<T>& nb, const OpRaw<T, OPK>& o, T) {
+    const T wv = op_apply<T, OPK, NDIM>(cf, o, nb);
     acc[0] += widen(nb.c) * widen(wv);
+    return wv;
+  }
+  __device__ __forceinline__ void operator()(long long idx, const Nbr<T>& nb, const Raw& q, int, int, int) {
+    w[idx] = value(nb, q.o, T(0));
     if constexpr (XUPD && fx_op(OPK)) {
       x[idx] = fma(ax, q.p, q.x);
     } else if constexpr (XUPD) {
@@ -323,6 +336,40 @@ __device__ BodyOut cg_body(const CgArgs<T>& a, const Team& tm, T* sm, double* sh
       // ---- pass 2: x += alpha p ; r -= alpha A p ; r.r
       const T tax = (T)(ar / a.sigma);      // multiplies p
       long long i = tm.tid();
+      if constexpr (CX == CX_QUAD) {
+        // four elements a lane (N is a multiple of 4), two quads in flight
+        const float4 *p4 = (const float4*)pnew, *w4 = (const float4*)a.w;
+        float4 *x4 = (float4*)a.x, *r4 = (float4*)a.r;
+        const long long N4 = N >> 2;
+        for (; i < N4; i += 2 * st) {
+          float4 pv[2], wv[2], xv[2], rv[2];
+#pragma unroll
+          for (int u = 0; u < 2; u++) {
+            const long long q = i + u * st < N4 ? i + u * st : i;
+            pv[u] = __ldcg(p4 + q);
+            wv[u] = __ldcg(w4 + q);
+            xv[u] = __ldcg(x4 + q);
+            rv[u] = __ldcg(r4 + q);
+          }
+#pragma unroll
+          for (int u = 0; u < 2; u++) {
+            if (u > 0 && i + st >= N4) break;
+            const long long q = i + u * st;
+            xv[u] = make_float4(fma(tax, pv[u].x, xv[u].x), fma(tax, pv[u].y, xv[u].y), fma(tax, pv[u].z, xv[u].z),
+                                fma(tax, pv[u].w, xv[u].w));
+            rv[u] = make_float4(fma(-tar, wv[u].x, rv[u].x), fma(-tar, wv[u].y, rv[u].y), fma(-tar, wv[u].z, rv[u].z),
+                                fma(-tar, wv[u].w, rv[u].w));
+            x4[q] = xv[u];
+            r4[q] = rv[u];
+            const double d0 = widen(rv[u].x), d1 = widen(rv[u].y), d2 = widen(rv[u].z), d3 = widen(rv[u].w);
+            acc1[0] += d0 * d0;
+            acc1[0] += d1 * d1;
+            acc1[0] += d2 * d2;
+            acc1[0] += d3 * d3;
+          }
+        }
+        i = N;   // nothing left for the loops below
+      }
       for (; i + (ILP - 1) * st < N; i += ILP * st) {
         T pv[ILP], wv[ILP], xv[ILP], rv[ILP];
 #pragma unroll
@@ -737,6 +784,17 @@ inline Coef<T> scaled_coef(const hs_op* A, double* sigma) {
   if (A->kind == KIND_HPCG27) cf.d = (T)(c.d + 1.0);
   if constexpr (std::is_same<T, double>::value) fx_weights(A, &cf.fx);
   return cf;
+}
+
+// Whether a solve takes the FP32 engine with four nodes per lane: x-lines of
+// whole quads (every vector is 16-byte aligned) that fill at least three
+// quarters of its 64-node tiles, rows per tile not chosen by the caller, and
+// at least 2^17 nodes.  us per iteration or sweep, one-node engine / quads: CG on
+// stored coefficients 64^3 22.8 / 19.3, 96^3 36.1 / 28.3, 128^3 46.9 / 33.9,
+// 192^3 101 / 79.9; Jacobi 64^3 6.2 / 6.1, 128^3 12.5 / 10.6, 192^3 28.4 / 19.1.
+inline bool quad_applies(const Geom& g, const hs_opts& o) {
+  const int wide = (g.nx + QTW - 1) / QTW * QTW;
+  return g.nx % 4 == 0 && 4 * g.nx >= 3 * wide && o.tile_rows == 0 && g.nz > 1 && g.N >= (1 << 17);
 }
 
 inline int rows_per_tile(const Geom& g) {

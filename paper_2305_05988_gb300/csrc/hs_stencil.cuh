@@ -114,10 +114,20 @@ template <int NDIM, class Src, class Sink>
 __device__ __forceinline__ void zmarch_fx(const Geom& g, const Tiling& tl, int item, double* sm, const Src& src,
                                            Sink& sink);
 
+// CX_QUAD selects the FP32 engine with four nodes per lane (hs_quad.cuh).
+constexpr int CX_QUAD = 4;
+template <class Src, class Sink>
+__device__ __forceinline__ void zmarch_quad(const Geom& g, const Tiling& tl, int item, float* sm, const Src& src,
+                                            Sink& sink);
+
 template <typename T, int NDIM, int CX, class Src, class Sink>
 __device__ __forceinline__ void zmarch_item(const Geom& g, const Tiling& tl, int item, T* sm, const Src& src,
                                             Sink& sink) {
-  if constexpr (is_box_sink<Sink>::value) {
+  if constexpr (CX == CX_QUAD) {
+    static_assert(std::is_same<T, float>::value && NDIM == 3, "the quad engine is FP32 and 3-D");
+    zmarch_quad(g, tl, item, sm, src, sink);
+    return;
+  } else if constexpr (is_box_sink<Sink>::value) {
     static_assert(NDIM == 3 && CX == 1, "the 27-point engine is 3-D with one column per lane");
     zmarch_box<T>(g, tl, item, sm, src, sink);
     return;
@@ -622,6 +632,7 @@ struct LoadSrc {
   __device__ __forceinline__ T make(const Raw& r, long long, bool) const { return r.v; }
   __device__ __forceinline__ const T* arr(int) const { return x; }
   __device__ __forceinline__ Raw pack(const T (&v)[1]) const { return Raw{v[0]}; }
+  __device__ __forceinline__ void put4(long long, const float4&) const {}
 };
 
 // ---------------------------------------------------------------------------
