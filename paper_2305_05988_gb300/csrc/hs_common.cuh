@@ -154,6 +154,9 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
+__device__ __forceinline__ void red_release(unsigned* p, unsigned v) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
 __device__ __forceinline__ void st_release(unsigned* p, unsigned v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
@@ -169,14 +172,14 @@ __device__ __forceinline__ int ld_acquire_int(const int* p) {
 // Control block at the start of every solver workspace (zeroed by the host
 // before each solve).
 struct Ctrl {
-  unsigned count;        // blocks arrived at the current barrier
-  unsigned gen;          // barrier generation
+  unsigned count;        // arrivals at the team's barriers (only grows; BatchTeam: at this one)
+  unsigned gen;          // barrier generation (BatchTeam)
   int status;            // DevStatus
   int iters;             // iterations completed
   int restarts;          // BiCGStab restarts
   int pad0;
   unsigned long long timeout_ns;
-  double scal[16];       // reduced scalars of the last barrier
+  double scal[16];       // reduced scalars of the last barrier (BatchTeam)
   double rel_res;        // last relative residual
   double aux[7];
 };
@@ -187,16 +190,31 @@ static_assert(sizeof(Ctrl) <= 512, "Ctrl must fit its 512-byte slot");
 // within the team, and the team's own control block and partial-sum slots.
 // A standalone solve uses the whole grid as one team; the batched solver runs
 // many teams (one per large system, single-block teams for small ones) in
-// one cooperative launch.
+// one cooperative launch.  A shared word of the block counts the grid team's
+// barriers since its control block was initialised (a register a thread would
+// cost the FP32 kernels a block per SM).
+constexpr int RED_MAX = 3;                 // scalars per reduction
+constexpr int RED_SLOTS = 2 * RED_MAX;     // partial sums per block (two barriers' worth)
+
 struct Team {
   int rank;
   int size;
   Ctrl* ctrl;
-  double* partials;   // size * NS doubles
+  double* partials;   // RED_SLOTS * size doubles
   __device__ __forceinline__ long long tid() const { return (long long)rank * blockDim.x + threadIdx.x; }
   __device__ __forceinline__ long long stride() const { return (long long)size * blockDim.x; }
   __device__ __forceinline__ bool lead() const { return rank == 0 && threadIdx.x == 0; }
 };
+
+__device__ __forceinline__ unsigned& team_epoch() {
+  __shared__ unsigned epoch;
+  return epoch;
+}
+// Before the first barrier of a grid team; the block barriers of a
+// reduction's block_sum come in between.
+__device__ __forceinline__ void team_begin() {
+  if (threadIdx.x == 0) team_epoch() = 0u;
+}
 
 __device__ __forceinline__ Team grid_team(Ctrl* ctrl, double* partials) {
   Team t;
@@ -204,21 +222,79 @@ __device__ __forceinline__ Team grid_team(Ctrl* ctrl, double* partials) {
   t.size = gridDim.x;
   t.ctrl = ctrl;
   t.partials = partials;
+  team_begin();
   return t;
 }
 
 // Team reduce-barrier.  Every block of the team contributes NS partial sums
-// (already block-reduced, valid in thread 0), the last block to arrive sums
-// all partials in rank order (so the result does not depend on arrival order),
-// publishes them in ctrl->scal and releases the others.  All threads of all
-// team blocks return the same NS doubles in `out`.  Returns false if the wait
-// ran out (ctrl->status is then DS_TIMEOUT) or another block flagged an error;
-// the caller must then stop working on this team's solve.
+// (block-reduced, valid in every thread), arrives on a counter that only
+// grows, waits until the whole team has arrived and sums all partials itself
+// in rank order, so the result does not depend on arrival order and is the
+// same in every block.  Three trips to L2 lie on the critical path (arrive,
+// see the count, read the partials); having the last block sum and release
+// the others took six.  A block one barrier ahead writes the other half of
+// the slots; it cannot be two ahead.  Returns false if the wait ran out
+// (ctrl->status is then DS_TIMEOUT) or another block flagged an error; the
+// caller must then stop working on this team's solve.
 //
 // All blocks of the team must be co-resident (cooperative launch).  `sh` needs
-// 32 * NS doubles of shared memory.
+// 32 * NS doubles of shared memory.  Not inlined: inlined, its loop costs the
+// stencil passes around it registers (FP32 CG on stored coefficients: 76 bytes
+// of spills instead of none, 285 instead of 210 us per iteration at 256^3).
 template <int NS>
-__device__ bool team_reduce(const Team& tm, const double (&mine)[NS], double (&out)[NS], double* sh) {
+__device__ __noinline__ bool team_reduce(const Team& tm, const double (&mine)[NS], double (&out)[NS], double* sh) {
+  static_assert(NS <= RED_MAX, "partial-sum slots");
+  __shared__ int s_ok;
+  const int tid = threadIdx.x;
+  Ctrl* ctrl = tm.ctrl;
+  const unsigned epoch = team_epoch();
+  double* slots = tm.partials + (size_t)(epoch & 1u) * RED_MAX * tm.size;
+  if (tid == 0) {
+#pragma unroll
+    for (int s = 0; s < NS; s++) slots[(size_t)tm.rank * NS + s] = mine[s];
+    red_release(&ctrl->count, 1u);
+    const unsigned target = (epoch + 1u) * (unsigned)tm.size;   // compared modulo 2^32
+    int ok = 1;
+    unsigned long long t0 = 0;
+    unsigned spins = 0;
+    while ((int)(ld_acquire(&ctrl->count) - target) < 0) {
+      if (++spins > 64) {
+        __nanosleep(100);
+        if ((spins & 255) == 0) {
+          if (t0 == 0) t0 = global_ns();
+          if (ld_acquire_int(&ctrl->status) < 0) { ok = 0; break; }
+          if (global_ns() - t0 > ctrl->timeout_ns) {
+            atomicCAS(&ctrl->status, 0, (int)DS_TIMEOUT);
+            ok = 0;
+            break;
+          }
+        }
+      }
+    }
+    s_ok = ok;
+  }
+  __syncthreads();
+  if (!s_ok) return false;
+  if (tid == 0) team_epoch() = epoch + 1u;
+#pragma unroll
+  for (int s = 0; s < NS; s++) out[s] = 0.0;
+  for (int b = tid; b < tm.size; b += blockDim.x) {
+#pragma unroll
+    for (int s = 0; s < NS; s++) out[s] += __ldcg(&slots[(size_t)b * NS + s]);
+  }
+  block_sum<NS>(out, sh);
+  return true;
+}
+
+// The teams of a batch: the last block to arrive sums the partials in rank
+// order, publishes the sums and releases the others.  Six trips to L2 instead
+// of three, but fewer registers and loads in the batch kernels, which spill
+// already (48 systems of 16 to 24 nodes a side, 40 iterations: 4.10 ms against
+// 4.64 with team_reduce above; up to 128 a side: 27.1 against 27.7).
+struct BatchTeam : Team {};
+
+template <int NS>
+__device__ bool team_reduce(const BatchTeam& tm, const double (&mine)[NS], double (&out)[NS], double* sh) {
   __shared__ int s_last;
   __shared__ int s_ok;
   Ctrl* ctrl = tm.ctrl;
@@ -283,20 +359,14 @@ __device__ bool team_reduce(const Team& tm, const double (&mine)[NS], double (&o
   return true;
 }
 
-// Whole-grid forms used by the standalone solver kernels.
-template <int NS>
-__device__ __forceinline__ bool grid_reduce(Ctrl* ctrl, double* partials, const double (&mine)[NS],
-                                            double (&out)[NS], double* sh) {
-  return team_reduce<NS>(grid_team(ctrl, partials), mine, out, sh);
-}
-
-// Plain barriers (no data).
-__device__ __forceinline__ bool team_sync(const Team& tm, double* sh) {
+// A plain barrier (no data).  The block barrier first: one thread arrives for
+// the block, which must not be before the other warps' work is done
+// (team_reduce's callers come from block_sum, which ends with one).
+template <class TM>
+__device__ __forceinline__ bool team_sync(const TM& tm, double* sh) {
+  __syncthreads();
   double z[1] = {0.0}, o[1];
   return team_reduce<1>(tm, z, o, sh);
-}
-__device__ __forceinline__ bool grid_sync(Ctrl* ctrl, double* partials, double* sh) {
-  return team_sync(grid_team(ctrl, partials), sh);
 }
 
 }  // namespace hs

@@ -341,6 +341,7 @@ __global__ void __launch_bounds__(gs_threads<NDIM, W>()) k_gs(GsArgs<T> a) {
   double* sh = reinterpret_cast<double*>(smraw);
   const long long N = a.g.N;
 
+  const Team tm = grid_team(a.cm.ctrl, a.cm.partials);
   double acc[1] = {0.0};
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
     T bv = a.b[i];
@@ -355,7 +356,7 @@ __global__ void __launch_bounds__(gs_threads<NDIM, W>()) k_gs(GsArgs<T> a) {
   unsigned long long cbase = 0;
   block_sum<1>(acc, sh);
   double bb[1];
-  if (!grid_reduce<1>(a.cm.ctrl, a.cm.partials, acc, bb, sh)) return;
+  if (!team_reduce<1>(tm, acc, bb, sh)) return;
   if (bb[0] == 0.0) {
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x)
       a.x[i] = T(0);
@@ -370,7 +371,7 @@ __global__ void __launch_bounds__(gs_threads<NDIM, W>()) k_gs(GsArgs<T> a) {
   int done = 0, status = DS_CONVERGED;
   double rel = -1.0;
   if (a.tol > 0.0) {
-    if (!gs_residual<T, OPK, NDIM>(a, sm, sh, bb[0], &rel)) return;
+    if (!gs_residual<T, OPK, NDIM>(a, tm, sh, bb[0], &rel)) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) a.cm.hist[0] = rel;
     if (!(rel > a.tol)) status = isfinite(rel) ? DS_CONVERGED : DS_NONFINITE;
     else status = DS_MAXIT;
@@ -382,7 +383,7 @@ __global__ void __launch_bounds__(gs_threads<NDIM, W>()) k_gs(GsArgs<T> a) {
         return;
       done += nb;
       if (a.tol > 0.0) {
-        if (!gs_residual<T, OPK, NDIM>(a, sm, sh, bb[0], &rel)) return;
+        if (!gs_residual<T, OPK, NDIM>(a, tm, sh, bb[0], &rel)) return;
         if (blockIdx.x == 0 && threadIdx.x == 0) {
           for (int q = done - nb + 1; q < done; q++) a.cm.hist[q] = nan("");  // not evaluated
           a.cm.hist[done] = rel;
@@ -540,7 +541,7 @@ static hs_status gs_run_t(const SolveArgs& sa, hs_result* res, double* hist) {
     set_error("Gauss-Seidel kernel cannot be resident");
     return HS_ERR_CUDA;
   }
-  int grid = std::min(per_sm * sm_count(), MAX_BLOCKS);
+  int grid = std::min(per_sm * sm_count(), MAX_TEAM);
   if (sa.o.max_blocks > 0) grid = std::min(grid, sa.o.max_blocks);
   void* args[] = {&a};
   e = cudaLaunchCooperativeKernel((const void*)kern, dim3(grid), dim3(THREADS), args, smem, sa.stream);

@@ -305,6 +305,7 @@ template <typename T, int OPK, bool VEC>
 __global__ void __launch_bounds__(32 * GSP_WARPS, HS_GSP_MINB) k_gsp(GsArgs<T> a, GspArgs G) {
   __shared__ double sh[32 * MAX_SCAL];
   const long long N = a.g.N;
+  const Team tm = grid_team(a.cm.ctrl, a.cm.partials);
   double acc[1] = {0.0};
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
     T bv = a.b[i];
@@ -317,7 +318,7 @@ __global__ void __launch_bounds__(32 * GSP_WARPS, HS_GSP_MINB) k_gsp(GsArgs<T> a
   unsigned gsweep = 0;
   block_sum<1>(acc, sh);
   double bb[1];
-  if (!grid_reduce<1>(a.cm.ctrl, a.cm.partials, acc, bb, sh)) return;
+  if (!team_reduce<1>(tm, acc, bb, sh)) return;
   if (bb[0] == 0.0) {
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x)
       a.x[i] = T(0);
@@ -332,7 +333,7 @@ __global__ void __launch_bounds__(32 * GSP_WARPS, HS_GSP_MINB) k_gsp(GsArgs<T> a
   int done = 0, status = DS_CONVERGED;
   double rel = -1.0;
   if (a.tol > 0.0) {
-    if (!gs_residual<T, OPK, 3>(a, nullptr, sh, bb[0], &rel)) return;
+    if (!gs_residual<T, OPK, 3>(a, tm, sh, bb[0], &rel)) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) a.cm.hist[0] = rel;
     if (!(rel > a.tol)) status = isfinite(rel) ? DS_CONVERGED : DS_NONFINITE;
     else status = DS_MAXIT;
@@ -343,7 +344,7 @@ __global__ void __launch_bounds__(32 * GSP_WARPS, HS_GSP_MINB) k_gsp(GsArgs<T> a
       if (!gsp_batch<T, OPK, VEC>(a, G, a.mode == HS_GS_SYMMETRIC ? 2 * nb : nb, a.mode, gsweep)) return;
       done += nb;
       if (a.tol > 0.0) {
-        if (!gs_residual<T, OPK, 3>(a, nullptr, sh, bb[0], &rel)) return;
+        if (!gs_residual<T, OPK, 3>(a, tm, sh, bb[0], &rel)) return;
         if (blockIdx.x == 0 && threadIdx.x == 0) {
           for (int q = done - nb + 1; q < done; q++) a.cm.hist[q] = nan("");  // not evaluated
           a.cm.hist[done] = rel;
@@ -396,7 +397,7 @@ static bool gsp_fits_t(const hs_op* A, const hs_opts& o) {
     cudaGetLastError();
     return false;
   }
-  long long blocks = std::min<long long>((long long)per_sm * sm_count(), MAX_BLOCKS);
+  long long blocks = std::min<long long>((long long)per_sm * sm_count(), MAX_TEAM);
   if (o.max_blocks > 0) blocks = std::min<long long>(blocks, o.max_blocks);
   return np <= blocks * GSP_WARPS && np >= 12ll * sm_count();
 }
@@ -435,7 +436,7 @@ static hs_status gsp_run_t(const SolveArgs& sa, hs_result* res, double* hist) {
     set_error("Gauss-Seidel kernel cannot be resident");
     return HS_ERR_CUDA;
   }
-  int grid = std::min(per_sm * sm_count(), MAX_BLOCKS);
+  int grid = std::min(per_sm * sm_count(), MAX_TEAM);
   grid = std::min(grid, (G.NP + GSP_WARPS - 1) / GSP_WARPS);
   if (sa.o.max_blocks > 0) grid = std::min(grid, sa.o.max_blocks);
   grid = std::max(grid, 1);

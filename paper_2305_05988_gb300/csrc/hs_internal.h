@@ -137,7 +137,9 @@ struct Carve {
 };
 
 constexpr int MAX_BLOCKS = 4096;   // cap on persistent grid size
-constexpr int MAX_SCAL = 4;        // scalars per grid reduction
+constexpr int MAX_SCAL = 4;        // partial-sum slots per block; 32 * MAX_SCAL doubles of reduction scratch
+// persistent grids whose reductions fit those slots
+constexpr int MAX_TEAM = MAX_BLOCKS * MAX_SCAL / RED_SLOTS;
 
 struct Common {
   Ctrl* ctrl;

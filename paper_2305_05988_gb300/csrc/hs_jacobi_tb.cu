@@ -152,6 +152,7 @@ __global__ void __launch_bounds__(tb_threads<S>()) k_jacobi_tb(JacTbArgs<T> a) {
   __shared__ double sh[32 * MAX_SCAL];
   T* sm = reinterpret_cast<T*>(smraw);
   const long long N = a.g.N;
+  const Team tm = grid_team(a.cm.ctrl, a.cm.partials);
   double acc[1] = {0.0};
   for (long long i = gtid(); i < N; i += gstride()) {
     const T bv = a.b[i];
@@ -160,7 +161,7 @@ __global__ void __launch_bounds__(tb_threads<S>()) k_jacobi_tb(JacTbArgs<T> a) {
   }
   block_sum<1>(acc, sh);
   double bb[1];
-  if (!grid_reduce<1>(a.cm.ctrl, a.cm.partials, acc, bb, sh)) return;
+  if (!team_reduce<1>(tm, acc, bb, sh)) return;
   if (bb[0] == 0.0) {
     for (long long i = gtid(); i < N; i += gstride()) a.x0[i] = T(0);
     finish(a.cm.ctrl, DS_CONVERGED, 0, 0.0);
@@ -171,7 +172,7 @@ __global__ void __launch_bounds__(tb_threads<S>()) k_jacobi_tb(JacTbArgs<T> a) {
   for (int done = 0; done < a.sweeps;) {
     const int L = min(S, a.sweeps - done);
     for (int item = blockIdx.x; item < a.tl.items(); item += gridDim.x) tb_item<T, OPK, S>(a, item, L, src, dst, sm);
-    if (!grid_sync(a.cm.ctrl, a.cm.partials, sh)) return;
+    if (!team_sync(tm, sh)) return;
     done += L;
     T* tmp = const_cast<T*>(src);
     src = dst;
@@ -225,7 +226,7 @@ static hs_status jacobi_tb_t(const SolveArgs& sa, hs_result* res, double* hist) 
     set_error("temporally blocked Jacobi cannot be resident");
     return HS_ERR_CUDA;
   }
-  int grid = std::min(per_sm * sm_count(), MAX_BLOCKS);
+  int grid = std::min(per_sm * sm_count(), MAX_TEAM);
   if (sa.o.max_blocks > 0) grid = std::min(grid, sa.o.max_blocks);
   Tiling tl = choose_tiling(g, by, grid, false, sa.o.tile_planes, 1);
   grid = std::max(1, std::min(grid, tl.items()));

@@ -192,7 +192,9 @@ struct JacobiSink {
 template <typename T, int OPK, int NDIM, int CX>
 constexpr int jac_maxnreg() {
   if (CX == CX_QUAD) return HS_JACQ_MAXNREG;
-  return fx_op(OPK) && NDIM == 3 ? HS_JAC_ISO_MAXNREG : 128;
+  if (fx_op(OPK)) return NDIM == 3 ? HS_JAC_ISO_MAXNREG : 128;
+  if (OPK == OP_VARK) return sizeof(T) == 8 ? 80 : 128;   // FP64: three blocks per SM (230 us a sweep; two: 249)
+  return sizeof(T) == 4 ? 64 : 128;                       // FP32: four
 }
 
 template <typename T, int OPK, int NDIM, bool FUSE, int CX>
@@ -202,6 +204,7 @@ __global__ void __launch_bounds__(512) __maxnreg__((jac_maxnreg<T, OPK, NDIM, CX
   T* sm = reinterpret_cast<T*>(smraw);
   const long long N = a.g.N;
 
+  const Team tm = grid_team(a.cm.ctrl, a.cm.partials);
   double acc[1] = {0.0};
   for (long long i = gtid(); i < N; i += gstride()) {
     T bv = a.b[i];
@@ -210,7 +213,7 @@ __global__ void __launch_bounds__(512) __maxnreg__((jac_maxnreg<T, OPK, NDIM, CX
   }
   block_sum<1>(acc, sh);
   double bb[1];
-  if (!grid_reduce<1>(a.cm.ctrl, a.cm.partials, acc, bb, sh)) return;
+  if (!team_reduce<1>(tm, acc, bb, sh)) return;
   if (bb[0] == 0.0) {
     for (long long i = gtid(); i < N; i += gstride()) a.x0[i] = T(0);
     finish(a.cm.ctrl, DS_CONVERGED, 0, 0.0);
@@ -233,7 +236,7 @@ __global__ void __launch_bounds__(512) __maxnreg__((jac_maxnreg<T, OPK, NDIM, CX
     if constexpr (FUSE) {
       block_sum<1>(sink.acc, sh);
       double rr[1];
-      if (!grid_reduce<1>(a.cm.ctrl, a.cm.partials, sink.acc, rr, sh)) return;
+      if (!team_reduce<1>(tm, sink.acc, rr, sh)) return;
       double sc = (OPK == OP_VARK) ? 1.0 : a.dscale2;
       rel = sqrt(rr[0] * sc / bb[0]);
       if (blockIdx.x == 0 && threadIdx.x == 0) a.cm.hist[k] = rel;
@@ -248,7 +251,7 @@ __global__ void __launch_bounds__(512) __maxnreg__((jac_maxnreg<T, OPK, NDIM, CX
         break;
       }
     } else {
-      if (!grid_sync(a.cm.ctrl, a.cm.partials, sh)) return;
+      if (!team_sync(tm, sh)) return;
     }
     T* t = xs;
     xs = xd;
@@ -332,7 +335,6 @@ __global__ void __launch_bounds__(512) __maxnreg__((bi_maxnreg<T, OPK, NDIM>()))
 __global__ void k_init_ctrl(Ctrl* c, unsigned long long timeout_ns) {
   if (threadIdx.x == 0) {
     c->count = 0;
-    c->gen = 0;
     c->status = 0;
     c->iters = 0;
     c->restarts = 0;
@@ -692,6 +694,8 @@ __global__ void k_diag_team(Ctrl* ctrl, double* partials) {
   tm.size = 2;
   tm.ctrl = ctrl;
   tm.partials = partials;
+  team_begin();
+  __syncthreads();
   double z[1] = {0.0}, o[1];
   team_reduce<1>(tm, z, o, sh);
 }

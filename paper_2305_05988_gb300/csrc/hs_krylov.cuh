@@ -216,15 +216,25 @@ struct ApDotSink {
   const T* pold;
   T ax;
   double acc[1];
-  struct Raw {
-    OpRaw<T, OPK> o;
-    T x, p;   // fx_op with XUPD: staged by the engine
+  struct Staged : OpRaw<T, OPK> {
+    T x, p;
   };
-  static constexpr int NB = XUPD ? 1 : 0, kAux = XUPD ? 1 : 99;   // p_old is the source's operand 1
+  // fx_op with XUPD: x and p_old (the source's operand 1) staged by the engine
+  static constexpr bool kStaged = XUPD && fx_op(OPK);
+  using Raw = std::conditional_t<kStaged, Staged, OpRaw<T, OPK>>;
+  static constexpr int NB = XUPD ? 1 : 0, kAux = XUPD ? 1 : 99;
   __device__ __forceinline__ const T* opnd(int) const { return x; }
-  __device__ __forceinline__ Raw pack(const T (&v)[1], T p) const { return Raw{{}, v[0], p}; }
+  __device__ __forceinline__ Raw pack(const T (&v)[1], T p) const {
+    Raw r{};
+    if constexpr (kStaged) {
+      r.x = v[0];
+      r.p = p;
+    }
+    return r;
+  }
   __device__ __forceinline__ Raw fetch(long long idx, int i, int j, int k) const {
-    return Raw{op_fetch<T, OPK, NDIM>(cf, g, idx, i, j, k), T(0), T(0)};
+    if constexpr (kStaged) return Raw{};
+    else return op_fetch<T, OPK, NDIM>(cf, g, idx, i, j, k);
   }
   static constexpr int NQ = 0;
   __device__ __forceinline__ T* out() const { return w; }
@@ -234,7 +244,7 @@ struct ApDotSink {
     return wv;
   }
   __device__ __forceinline__ void operator()(long long idx, const Nbr<T>& nb, const Raw& q, int, int, int) {
-    w[idx] = value(nb, q.o, T(0));
+    w[idx] = value(nb, q, T(0));
     if constexpr (XUPD && fx_op(OPK)) {
       x[idx] = fma(ax, q.p, q.x);
     } else if constexpr (XUPD) {
@@ -251,8 +261,8 @@ struct ApDotSink {
 // (ApDotSink<XUPD>), leaving pass 2 with r alone.  It pays where pass 1 is
 // FP64-pipe bound (standalone FP64); FP32 passes are memory bound and the
 // batched kernel is register bound, so they keep x in pass 2.
-template <typename T, int OPK, int NDIM, int CX = cx_cg<T, OPK>(), bool XDEFER = false>
-__device__ BodyOut cg_body(const CgArgs<T>& a, const Team& tm, T* sm, double* sh) {
+template <typename T, int OPK, int NDIM, int CX = cx_cg<T, OPK>(), bool XDEFER = false, class TM = Team>
+__device__ BodyOut cg_body(const CgArgs<T>& a, const TM& tm, T* sm, double* sh) {
   const long long N = a.g.N;
   const T sig = (T)a.sigma;
 
@@ -587,8 +597,8 @@ struct BiTSink {
 };
 
 // The BiCGStab iteration run by one team of blocks.
-template <typename T, int OPK, int NDIM, int CX = CX_BI>
-__device__ BodyOut bicgstab_body(const BiArgs<T>& a, const Team& tm, T* sm, double* sh) {
+template <typename T, int OPK, int NDIM, int CX = CX_BI, class TM = Team>
+__device__ BodyOut bicgstab_body(const BiArgs<T>& a, const TM& tm, T* sm, double* sh) {
   const long long N = a.g.N;
   const T sig = (T)a.sigma;
 
@@ -840,7 +850,7 @@ inline hs_status plan_persistent(K kernel, int block, size_t smem, const Geom& g
     set_error("persistent kernel cannot be resident (block %d, smem %zu)", block, smem);
     return HS_ERR_CUDA;
   }
-  int grid = std::min(per_sm * sm_count(), MAX_BLOCKS);
+  int grid = std::min(per_sm * sm_count(), MAX_TEAM);
   if (o.max_blocks > 0) grid = std::min(grid, o.max_blocks);
   Tiling tl = choose_tiling(g, by, grid, src_expensive, o.tile_planes, cx);
   grid = std::max(1, std::min(grid, tl.items()));
