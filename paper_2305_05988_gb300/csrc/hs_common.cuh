@@ -216,8 +216,9 @@ __device__ __forceinline__ void team_begin() {
   if (threadIdx.x == 0) team_epoch() = 0u;
 }
 
-__device__ __forceinline__ Team grid_team(Ctrl* ctrl, double* partials) {
-  Team t;
+template <class TM = Team>
+__device__ __forceinline__ TM grid_team(Ctrl* ctrl, double* partials) {
+  TM t;
   t.rank = blockIdx.x;
   t.size = gridDim.x;
   t.ctrl = ctrl;
@@ -238,11 +239,9 @@ __device__ __forceinline__ Team grid_team(Ctrl* ctrl, double* partials) {
 // caller must then stop working on this team's solve.
 //
 // All blocks of the team must be co-resident (cooperative launch).  `sh` needs
-// 32 * NS doubles of shared memory.  Not inlined: inlined, its loop costs the
-// stencil passes around it registers (FP32 CG on stored coefficients: 76 bytes
-// of spills instead of none, 285 instead of 210 us per iteration at 256^3).
+// 32 * NS doubles of shared memory.
 template <int NS>
-__device__ __noinline__ bool team_reduce(const Team& tm, const double (&mine)[NS], double (&out)[NS], double* sh) {
+__device__ __forceinline__ bool team_reduce_impl(const Team& tm, const double (&mine)[NS], double (&out)[NS], double* sh) {
   static_assert(NS <= RED_MAX, "partial-sum slots");
   __shared__ int s_ok;
   const int tid = threadIdx.x;
@@ -284,6 +283,22 @@ __device__ __noinline__ bool team_reduce(const Team& tm, const double (&mine)[NS
   }
   block_sum<NS>(out, sh);
   return true;
+}
+
+// Called or inlined: inlined (InlineTeam), Jacobi and the FP64 neighbour-sum
+// kernels run faster (256^3 Jacobi 109 against 115 us per sweep, 250 x 187 x 141
+// 64 against 82, 128^2 BiCGStab 22.9 against 25.2); the other stencil passes
+// lose registers to it (FP32 CG on stored coefficients, one node per lane: 76
+// bytes of spills, 285 instead of 249 us per iteration).
+template <int NS>
+__device__ __noinline__ bool team_reduce(const Team& tm, const double (&mine)[NS], double (&out)[NS], double* sh) {
+  return team_reduce_impl<NS>(tm, mine, out, sh);
+}
+struct InlineTeam : Team {};
+template <int NS>
+__device__ __forceinline__ bool team_reduce(const InlineTeam& tm, const double (&mine)[NS], double (&out)[NS],
+                                            double* sh) {
+  return team_reduce_impl<NS>(tm, mine, out, sh);
 }
 
 // The teams of a batch: the last block to arrive sums the partials in rank

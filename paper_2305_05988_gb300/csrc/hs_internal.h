@@ -117,8 +117,9 @@ inline int kernel_op(const hs_op* A, hs_dtype dt) {
 }
 
 // Chooses a tiling (rows per tile, z chunk length) for `grid` persistent
-// blocks, or for a one-item-per-block launch when grid == 0.
-Tiling choose_tiling(const Geom& g, int by, int grid, bool src_expensive, int planes = 0, int cx = 1);
+// blocks sharing `sms` SMs (0: a team of a batch), or for a one-item-per-block
+// launch when grid == 0.
+Tiling choose_tiling(const Geom& g, int by, int grid, bool src_expensive, int planes = 0, int cx = 1, int sms = 0);
 
 // Workspace carving: every section is 256-byte aligned.
 struct Carve {

@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(512) __maxnreg__((jac_maxnreg<T, OPK, NDIM, CX
   T* sm = reinterpret_cast<T*>(smraw);
   const long long N = a.g.N;
 
-  const Team tm = grid_team(a.cm.ctrl, a.cm.partials);
+  const InlineTeam tm = grid_team<InlineTeam>(a.cm.ctrl, a.cm.partials);
   double acc[1] = {0.0};
   for (long long i = gtid(); i < N; i += gstride()) {
     T bv = a.b[i];
@@ -302,6 +302,7 @@ constexpr int cg_maxnreg() {
   if (fx_op(OPK) && NDIM == 3) return HS_CG_ISO_MAXNREG;
   if (sizeof(T) == 4) return (HS_CG32_MAXNREG > 0 && OPK == OP_VARK) ? HS_CG32_MAXNREG : 255;
   if (OPK == OP_VARK) return HS_CGV64_MAXNREG > 0 ? HS_CGV64_MAXNREG : 255;
+  if (OPK == OP_BOX27) return 72;   // 128 x 128 x 512: 278.8 us per iteration (64: 283.4, 80: 278.9)
   return HS_CG_MAXNREG > 0 ? HS_CG_MAXNREG : 255;
 }
 template <typename T, int OPK, int NDIM>
@@ -315,7 +316,8 @@ template <typename T, int OPK, int NDIM, int CX>
 __global__ void __launch_bounds__(512) __maxnreg__((cg_maxnreg<T, OPK, NDIM, CX>())) k_cg(CgArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ double sh[32 * MAX_SCAL];
-  const Team tm = grid_team(a.cm.ctrl, a.cm.partials);
+  using TM = std::conditional_t<fx_op(OPK), InlineTeam, Team>;
+  const TM tm = grid_team<TM>(a.cm.ctrl, a.cm.partials);
   constexpr bool xdefer = HS_CG_XDEFER && sizeof(T) == 8 && OPK != OP_VARK;
   team_finish(tm, cg_body<T, OPK, NDIM, CX, xdefer>(a, tm, reinterpret_cast<T*>(smraw), sh));
 }
@@ -324,7 +326,8 @@ template <typename T, int OPK, int NDIM>
 __global__ void __launch_bounds__(512) __maxnreg__((bi_maxnreg<T, OPK, NDIM>())) k_bicgstab(BiArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ double sh[32 * MAX_SCAL];
-  const Team tm = grid_team(a.cm.ctrl, a.cm.partials);
+  using TM = std::conditional_t<fx_op(OPK), InlineTeam, Team>;
+  const TM tm = grid_team<TM>(a.cm.ctrl, a.cm.partials);
   team_finish(tm, bicgstab_body<T, OPK, NDIM>(a, tm, reinterpret_cast<T*>(smraw), sh));
 }
 
@@ -354,7 +357,7 @@ int sm_count() {
   return g_sm_count;
 }
 
-Tiling choose_tiling(const Geom& g, int by, int grid, bool src_expensive, int planes, int cx) {
+Tiling choose_tiling(const Geom& g, int by, int grid, bool src_expensive, int planes, int cx, int sms) {
   Tiling t;
   t.by = by;
   t.cx = cx;
@@ -379,18 +382,30 @@ Tiling choose_tiling(const Geom& g, int by, int grid, bool src_expensive, int pl
   const double over = src_expensive ? 2.0 : 1.0;
   double best = 1e300;
   int best_lz = g.nz;
-  for (int lz = 4; lz <= g.nz; lz++) {
+  // Cost of a pass: items in turn on the busiest unit x (planes + the start of
+  // an item).  Small Krylov passes (up to 24 tile planes per SM): the unit is
+  // the SM, whose FP64 pipe and issue slots the resident blocks share (64^3 CG:
+  // 128 items of 8 planes, one per SM, 17.1 us per iteration; 256 of 4, two on
+  // most SMs, 21.6; 96^3 30 against 36).  Beyond, and for sweeps of plain loads,
+  // a block alone on its SM cannot fill it (192^3 CG 173 against 118), and in a
+  // batch other teams share the SM: the unit is the block, items of four planes
+  // at least.
+  if (!src_expensive || (long long)txy * g.nz > 24ll * sms) sms = 0;
+  const int lz_min = sms > 0 ? 1 : 4;
+  const int units = sms > 0 ? std::min(sms, grid) : grid;
+  const int per_unit = (grid + units - 1) / units;
+  for (int lz = lz_min; lz <= g.nz; lz++) {
     int chunks = (g.nz + lz - 1) / lz;
-    if (lz > 4 && (g.nz + lz - 2) / (lz - 1) == chunks) continue;  // same chunk count, smaller lz better
+    if (lz > lz_min && (g.nz + lz - 2) / (lz - 1) == chunks) continue;  // same chunk count, smaller lz better
     long long items = (long long)txy * chunks;
-    long long waves = (items + grid - 1) / grid;
-    double cost = (double)waves * (lz + over);
+    long long load = items <= grid ? (items + units - 1) / units : (items + grid - 1) / grid * per_unit;
+    double cost = (double)load * (lz + over);
     if (cost < best - 1e-9) {
       best = cost;
       best_lz = lz;
     }
   }
-  if (g.nz < 4) best_lz = g.nz;
+  if (sms <= 0 && g.nz < 4) best_lz = g.nz;
   t.lz = best_lz;
   t.chunks = (g.nz + t.lz - 1) / t.lz;
   return t;

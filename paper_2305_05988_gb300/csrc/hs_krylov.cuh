@@ -852,9 +852,14 @@ inline hs_status plan_persistent(K kernel, int block, size_t smem, const Geom& g
   }
   int grid = std::min(per_sm * sm_count(), MAX_TEAM);
   if (o.max_blocks > 0) grid = std::min(grid, o.max_blocks);
-  Tiling tl = choose_tiling(g, by, grid, src_expensive, o.tile_planes, cx);
-  grid = std::max(1, std::min(grid, tl.items()));
-  *tl_out = choose_tiling(g, by, grid, src_expensive, o.tile_planes, cx);
+  *tl_out = choose_tiling(g, by, grid, src_expensive, o.tile_planes, cx, sm_count());
+  grid = std::max(1, std::min(grid, tl_out->items()));
+  // blocks that would sit out the last round of items are not launched, unless
+  // that takes more than one in 32 from the elementwise passes (256^3 BiCGStab:
+  // 448 blocks of exactly four items instead of 456)
+  const int rounds = (tl_out->items() + grid - 1) / grid;
+  const int even = (tl_out->items() + rounds - 1) / rounds;
+  if (32 * even >= 31 * grid) grid = even;
   *grid_out = grid;
   return HS_OK;
 }
