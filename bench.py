@@ -49,26 +49,27 @@ BYTES = {
     "bicgstab": 136.0,     # per iteration (17 vector passes of 8 B)
 }
 
-# FP64 flops per unknown and iteration executed by the kernels (FMA = 2),
-# counted from the kernel code for the 7-point operators of the workload:
-#   spmv      3 pair adds + 3 FMA + 1 scaling multiply             = 10
-#   jacobi    3 pair adds + 3 FMA                                   =  9
-#   gs        as jacobi                                             =  9
-#   cg        p update FMA, stencil 3 adds + 3 FMA, p.w FMA;
-#             x and r FMA, r.r FMA                                  = 19
-#   bicgstab  p update 2 FMA, upwind stencil 6 FMA, v.r' FMA;
-#             s FMA, stencil 6 FMA, 3 dot FMA; x 2 FMA, r FMA,
-#             2 dot FMA                                             = 48
-FLOPS = {"spmv": 10.0, "jacobi": 9.0, "gauss_seidel": 9.0, "cg": 19.0, "bicgstab": 48.0}
+# FP64 flops per unknown and iteration executed on the FP64 pipe (FMA = 2),
+# counted from the kernel code for the 7-point operators of the workload (the
+# neighbour sums run on the integer pipes, except in Gauss-Seidel):
+#   spmv      1 FMA + 1 scaling multiply                            =  3
+#   jacobi    1 FMA                                                 =  2
+#   gs        3 pair adds + 3 FMA                                   =  9
+#   cg        p update FMA, stencil 1 FMA, p.w FMA;
+#             x and r FMA, r.r FMA                                  = 12
+#   bicgstab  p update 2 FMA, stencil 1 FMA, v.r' FMA;
+#             s FMA, stencil 1 FMA, 3 dot FMA; x 2 FMA, r FMA,
+#             2 dot FMA                                             = 28
+FLOPS = {"spmv": 3.0, "jacobi": 2.0, "gauss_seidel": 9.0, "cg": 12.0, "bicgstab": 28.0}
 
 # DRAM bytes per unknown and iteration measured by ncu (dram__bytes_read.sum +
 # dram__bytes_write.sum) on short launches of the same kernels at 256^3
-# (profiles/fp64_and_traffic_poisson3d_256.md: CG and BiCGStab 10 iterations,
+# (profiles/neighbour_sums_poisson3d_256.md: CG and BiCGStab 10 iterations,
 # Jacobi 20 sweeps, one launch per capture; the start-up residual pass is
 # subtracted).  Traffic grows with unknowns x iterations (each pass streams
 # every vector), so a launch of the step moves this figure x N x iterations.
 # Re-measure whenever the kernel changes.
-TRAFFIC_B_PER_UNIT = {"cg": 74.3, "bicgstab": 135.1, "jacobi": 24.9}
+TRAFFIC_B_PER_UNIT = {"cg": 74.8, "bicgstab": 138.8, "jacobi": 25.2}
 # FP64 pipe: 2 FMA lanes per SM per clock (ncu: sm__sass_thread_inst_executed_op_dfma_pred_on
 # peak_sustained = 2 per SM per cycle) x 2 flops x 152 SMs.
 FP64_FLOPS_PER_CLK = 2 * 2 * 152

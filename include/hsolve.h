@@ -99,7 +99,9 @@ typedef struct {
     int tile_rows;          /* stencil tiles of the Jacobi / CG / BiCGStab /
                                mixed solvers: rows of 32 nodes per tile = warps
                                per block, 4 to 16 (other values: the built-in
-                               heuristic, 8 rows on 3-D grids)                 */
+                               heuristic, 8 rows on 3-D grids; 64 x 16 nodes
+                               for FP32 Jacobi and CG on large 3-D grids with
+                               n_x a multiple of 4)                            */
     int tile_planes;        /* z planes per work item of those tiles; 0 = the
                                built-in cost model                             */
     int max_blocks;         /* cap on the persistent grid (blocks); 0 = all

@@ -6,7 +6,7 @@
 // cheaper as a fixed-point sum: each term is split once into a signed 60-bit
 // significand and its exponent (fx_make), the terms are shifted to the largest
 // exponent of the sum, added as 64-bit integers and rounded once to binary64
-// (fx_total).  Six terms take 42 cycles per warp and sub-partition, a split 8
+// (fx_total).  Six terms take about 42 cycles per warp and sub-partition, a split 8
 // (measured at full occupancy); five FP64 additions take 320.
 //
 // Accuracy: a term loses less than 2^-59 of the largest term's power of two
