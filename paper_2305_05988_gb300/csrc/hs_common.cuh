@@ -58,13 +58,13 @@ enum DevStatus : int {
 //
 // FxW: the couplings of an OP_WSYM / OP_WNON operator relative to the upper x
 // one, in the order xl, xu, yl, yu, zl, zu: as doubles w, and as fixed-point
-// fractions of 2^k, c = w 2^(62 - k) < 2^61 in limbs of 31 bits (ch, cl);
-// rc = the rounding constant of a product (see fx_scale).
+// significand and exponent, w = c 2^(x - 60), 2^60 <= c < 2^61 in limbs of 31
+// bits (ch, cl); rc = the rounding constant of a product (see fx_scale).
 struct FxW {
   double w[6];
   int ch[6], cl[6];
   unsigned rc[6];
-  int k;
+  int x[6];
 };
 
 template <typename T>

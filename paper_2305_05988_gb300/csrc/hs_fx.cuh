@@ -10,12 +10,16 @@
 // (measured at full occupancy); five FP64 additions take 320.
 //
 // Accuracy: a term loses less than 2^-59 of the largest term's power of two
-// when it is shifted, so n <= 7 terms are summed to within 7 x 2^-59 of it
-// before the one rounding (weighted sums: 6 x 2^-57 of the largest weighted
-// one); a chain of FP64 additions rounds n - 1 times at
-// 2^-53 of its partial sums.  Sums that cancel below 2^-16 of the largest
-// term, terms outside 2^-943 .. 2^1006 and non-finite terms take the FP64
-// additions themselves (fx_value restores every double exactly, zeros,
+// when it is shifted by more than seven places (up to there the shift is
+// exact), always towards minus infinity, so n <= 7 terms are summed to within
+// 7 x 2^-59 of it before the one rounding.  Weighted terms are aligned by the
+// exponent of the weighted term, so their error is relative to the largest
+// weighted term too, however far the weights lie apart: 4.5 x 2^-56 of its
+// power of two for three pairs, 7.5 x 2^-56 for six single terms
+// (fx_neighbours).  A chain of FP64 additions rounds n - 1 times at 2^-53 of
+// its partial sums.  Sums that cancel below 2^-16 (weighted: 2^-12) of the
+// largest term, terms outside 2^-943 .. 2^1006 and non-finite terms take the
+// FP64 additions themselves (fx_value restores every double exactly, zeros,
 // subnormals, infinities and NaNs included).
 #pragma once
 #include <cuda_runtime.h>
@@ -78,10 +82,10 @@ __device__ __forceinline__ bool fx_round(long long acc, unsigned top, double& y)
   return true;
 }
 
-// The significand shifted to the exponent top >= f.e.
-__device__ __forceinline__ long long fx_align(const Fx& f, unsigned top) {
+// The significand shifted right.
+__device__ __forceinline__ long long fx_align(const Fx& f, unsigned by) {
   long long m = ((long long)f.hi << 32) | f.lo;
-  asm("shr.s64 %0, %0, %1;" : "+l"(m) : "r"(top - f.e));   // amounts above 63 leave the sign
+  asm("shr.s64 %0, %0, %1;" : "+l"(m) : "r"(by));   // amounts above 63 leave the sign
   return m;
 }
 
@@ -100,7 +104,7 @@ __device__ __forceinline__ double fx_total(const Fx (&v)[n]) {
   const unsigned top = fx_top(v);
   long long acc = 0;
 #pragma unroll
-  for (int q = 0; q < n; q++) acc += fx_align(v[q], top);
+  for (int q = 0; q < n; q++) acc += fx_align(v[q], top - v[q].e);
   double y;
   if (fx_round(acc, top, y)) return y;
   y = fx_value(v[0]);
@@ -124,25 +128,49 @@ __device__ __forceinline__ long long fx_scale(long long m, const FxW& W, int q) 
 }
 
 // The sum of a node's neighbours in the order w, e, s, n, b, t, weighted by
-// the couplings relative to the upper x one (OP_WSYM, OP_WNON).  Terms are
-// aligned first (exact for exponents up to 7 apart), then scaled with
-// rounding to 2^-57 of the largest coupling's term.
+// the couplings relative to the upper x one (OP_WSYM, OP_WNON).
+//
+// Coupling q is (c_q / 2^60) 2^(x_q) with c_q in [2^60, 2^61), so the weighted
+// term's exponent is e + x_q, up to the last bit; terms are shifted to the
+// largest of those and the products summed in units of 2^-56 of that power of
+// two.  A product is off by one unit at most (fx_scale: half for the rounding,
+// half for the mean), the shift in front of it by a quarter (a pair: half).
+// Aligned by e alone, as in OP_ISO, the unit would be relative to the largest
+// value times the largest coupling: at a ratio of 62 a single neighbour on the
+// weak axis came out wrong by 5.9 x 2^-53, and by up to 25 x 2^-53 of the terms next to small
+// neighbours on the strong axes, where FP64 additions stay below 1.5.
 template <int OPK, int n>
 __device__ __forceinline__ double fx_neighbours(const Fx (&v)[n], const FxW& W) {
   if constexpr (OPK == OP_ISO) {
     return fx_total(v);
   } else {
-    const unsigned top = fx_top(v);
+    // W.x[1], and in OP_WSYM W.x[0], is zero: the upper x weight is 1.  (The
+    // two forms: 250 x 187 x 141 Jacobi, OP_WSYM, 72.0 us per sweep against 73.3
+    // in the other; 256^3, OP_WNON, 176.8 against 181.5.)
+    int top;
     long long acc = 0;
     if constexpr (OPK == OP_WSYM) {
+      top = max((int)v[0].e, (int)v[1].e);
 #pragma unroll
-      for (int q = 0; q < n; q += 2) acc += fx_scale(fx_align(v[q], top) + fx_align(v[q + 1], top), W, q);
+      for (int q = 2; q < n; q++) top = __viaddmax_s32((int)v[q].e, W.x[q], top);
+#pragma unroll
+      for (int q = 0; q < n; q += 2) {
+        const unsigned at = (unsigned)(q == 0 ? top : top - W.x[q]);
+        acc += fx_scale(fx_align(v[q], at - v[q].e) + fx_align(v[q + 1], at - v[q + 1].e), W, q);
+      }
     } else {
+      int e[n];
+      top = -64;
 #pragma unroll
-      for (int q = 0; q < n; q++) acc += fx_scale(fx_align(v[q], top), W, q);
+      for (int q = 0; q < n; q++) {
+        e[q] = (int)v[q].e + (q == 1 ? 0 : W.x[q]);
+        top = max(top, e[q]);
+      }
+#pragma unroll
+      for (int q = 0; q < n; q++) acc += fx_scale(fx_align(v[q], (unsigned)(top - e[q])), W, q);
     }
     double y;
-    if (fx_round(acc, top, y)) return __hiloint2double(__double2hiint(y) + ((W.k + 1) << 20), __double2loint(y));
+    if (fx_round(acc, (unsigned)top, y)) return __hiloint2double(__double2hiint(y) + (3 << 20), __double2loint(y));
     y = W.w[0] * fx_value(v[0]);
 #pragma unroll
     for (int q = 1; q < n; q++) y = fma(W.w[q], fx_value(v[q]), y);

@@ -102,9 +102,9 @@ bool fx_weights(const hs_op* A, FxW* W);
 
 // The operator kind a kernel is compiled for.  FP64 operators in 2-D and 3-D
 // take the neighbour sum on the integer pipes where the couplings lie within
-// a factor of 64 (grid spacings within 8, cell Peclet numbers to 31): beyond,
-// the fixed-point products would be coarser than FP64's rounding for the
-// weakest coupling.
+// a factor of 64 (grid spacings within 8, cell Peclet numbers to 31).  The
+// error of the sums does not depend on the factor (fx_neighbours); up to there
+// they are tested against extended precision and timed.
 inline int kernel_op(const hs_op* A, hs_dtype dt) {
   const int opk = opkind_of(A);
   if ((opk != OP_SYM && opk != OP_NONSYM) || dt != HS_F64 || A->ndim < 2) return opk;

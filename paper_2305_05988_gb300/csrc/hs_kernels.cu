@@ -444,12 +444,10 @@ bool fx_weights(const hs_op* A, FxW* W) {
     hi = std::max(hi, W->w[q]);
   }
   if (!(hi <= 64.0 * lo)) return false;
-  // 2^k > 2 max w, so that c = w 2^(62 - k) < 2^61; within a factor of 64 every
-  // c is exact
-  std::frexp(hi, &W->k);
-  W->k += 1;
   for (int q = 0; q < 2 * A->ndim; q++) {
-    const long long v = (long long)std::ldexp(W->w[q], 62 - W->k);
+    int k;
+    const long long v = (long long)std::ldexp(std::frexp(W->w[q], &k), 61);   // exact: 53 significant bits
+    W->x[q] = k - 1;
     W->ch[q] = (int)(v >> 31);
     W->cl[q] = (int)(v & 0x7fffffff);
     W->rc[q] = 0x80000000u + (unsigned)W->cl[q];
