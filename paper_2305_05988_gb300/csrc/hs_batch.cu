@@ -90,7 +90,7 @@ __device__ __forceinline__ void batch_job(const BatchSys* __restrict__ sys, int 
     for (int w = threadIdx.x; w < (int)(sizeof(BatchSys) / 8); w += blockDim.x) dst[w] = src[w];
   }
   __syncthreads();
-  BatchTeam tm;
+  LastTeam tm;
   tm.rank = rank;
   tm.size = size;
   tm.ctrl = sys_ctrl(d);

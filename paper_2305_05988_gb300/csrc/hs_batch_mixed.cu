@@ -52,11 +52,11 @@ __device__ __forceinline__ double pow2_inverse(double v) {
 }
 
 template <int OPK, int NDIM, bool BI>
-__device__ void mx_body(MxSys& a, const BatchTeam& tm, unsigned char* smraw, double* sh) {
+__device__ void mx_body(MxSys& a, const LastTeam& tm, unsigned char* smraw, double* sh) {
   double* sm64 = reinterpret_cast<double*>(smraw);
   float* sm32 = reinterpret_cast<float*>(smraw);
   const long long N = a.g.N;
-  BatchTeam ti = tm;
+  LastTeam ti = tm;
   ti.ctrl = a.inner_ctrl;
 
   // d = 0 and the scale of the first residual (from the RMS of b)
@@ -158,7 +158,7 @@ __device__ __forceinline__ void mx_job(const MxSys* __restrict__ sys, int s, int
     for (int w = threadIdx.x; w < (int)(sizeof(MxSys) / 8); w += blockDim.x) dst[w] = src[w];
   }
   __syncthreads();
-  BatchTeam tm;
+  LastTeam tm;
   tm.rank = rank;
   tm.size = size;
   tm.ctrl = d.cm.ctrl;

@@ -371,6 +371,7 @@ __global__ void __launch_bounds__(32 * (BY + 1), HS_CG32V_MINB) k_cg32v(const __
   extern __shared__ unsigned char smraw[];
   __shared__ double sh[32 * MAX_SCAL];
   unsigned char* base = reinterpret_cast<unsigned char*>(((uintptr_t)smraw + 127) & ~(uintptr_t)127);
+  team_begin();
   const Team tm = grid_team(a.cm.ctrl, a.cm.partials);
   Engine<BY> E;
   E.ring = base;

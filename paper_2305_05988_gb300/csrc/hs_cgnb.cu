@@ -139,6 +139,7 @@ __global__ void __launch_bounds__(512) k_cg_nb(CgnbArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ double sh[32 * MAX_SCAL];
   T* sm = reinterpret_cast<T*>(smraw);
+  team_begin();
   const Team tm = grid_team(a.cm.ctrl, a.cm.partials);
   const long long N = a.g.N;
   const long long st = tm.stride();

@@ -157,6 +157,11 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
 __device__ __forceinline__ void red_release(unsigned* p, unsigned v) {
   asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
+__device__ __forceinline__ unsigned atom_acq_rel(unsigned* p, unsigned v) {
+  unsigned r;
+  asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(r) : "l"(p), "r"(v) : "memory");
+  return r;
+}
 __device__ __forceinline__ void st_release(unsigned* p, unsigned v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
@@ -172,14 +177,14 @@ __device__ __forceinline__ int ld_acquire_int(const int* p) {
 // Control block at the start of every solver workspace (zeroed by the host
 // before each solve).
 struct Ctrl {
-  unsigned count;        // arrivals at the team's barriers (only grows; BatchTeam: at this one)
-  unsigned gen;          // barrier generation (BatchTeam)
+  unsigned count;        // arrivals at the team's barriers (only grows; LastTeam: at this one)
+  unsigned gen;          // barrier generation (LastTeam)
   int status;            // DevStatus
   int iters;             // iterations completed
   int restarts;          // BiCGStab restarts
   int pad0;
   unsigned long long timeout_ns;
-  double scal[16];       // reduced scalars of the last barrier (BatchTeam)
+  double scal[16];       // reduced scalars of the last barrier (LastTeam)
   double rel_res;        // last relative residual
   double aux[7];
 };
@@ -200,7 +205,7 @@ struct Team {
   int rank;
   int size;
   Ctrl* ctrl;
-  double* partials;   // RED_SLOTS * size doubles
+  double* partials;   // RED_SLOTS * size doubles (LastTeam: NS * size)
   __device__ __forceinline__ long long tid() const { return (long long)rank * blockDim.x + threadIdx.x; }
   __device__ __forceinline__ long long stride() const { return (long long)size * blockDim.x; }
   __device__ __forceinline__ bool lead() const { return rank == 0 && threadIdx.x == 0; }
@@ -216,56 +221,66 @@ __device__ __forceinline__ void team_begin() {
   if (threadIdx.x == 0) team_epoch() = 0u;
 }
 
-template <class TM = Team>
-__device__ __forceinline__ TM grid_team(Ctrl* ctrl, double* partials) {
-  TM t;
-  t.rank = blockIdx.x;
-  t.size = gridDim.x;
-  t.ctrl = ctrl;
-  t.partials = partials;
-  team_begin();
-  return t;
-}
-
 // Team reduce-barrier.  Every block of the team contributes NS partial sums
-// (block-reduced, valid in every thread), arrives on a counter that only
-// grows, waits until the whole team has arrived and sums all partials itself
-// in rank order, so the result does not depend on arrival order and is the
-// same in every block.  Three trips to L2 lie on the critical path (arrive,
-// see the count, read the partials); having the last block sum and release
-// the others took six.  A block one barrier ahead writes the other half of
-// the slots; it cannot be two ahead.  Returns false if the wait ran out
-// (ctrl->status is then DS_TIMEOUT) or another block flagged an error; the
-// caller must then stop working on this team's solve.
+// (block-reduced, valid in every thread) and arrives on a counter that only
+// grows.  All partials are summed in rank order, so the result does not depend
+// on arrival order and is the same in every block:
+//   every form: each block waits for the whole team and sums them itself.
+//     Three trips to L2 lie on the critical path (arrive, see the count, read
+//     the partials), but size^2 NS values are read;
+//   last form: the last block to arrive sums them, publishes the sums and
+//     releases the others: six trips, size NS values.
+// us per barrier, every / last form: one scalar 152 blocks 2.5 / 4.6, 304 3.7 /
+// 5.4, 608 (the largest grid with one) 6.3 / 6.5; two 304 4.7 / 6.0, 456 6.7 /
+// 6.4, 608 8.5 / 7.3; three 304 5.7 / 7.3, 456 8.5 / 7.7, 608 10.9 / 8.7.  So
+// Team is always the every form, and BiTeam, for BiCGStab with its two and
+// three scalars in every iteration, takes the last form beyond 400 blocks (FP32
+// at 2048^2 168 us per iteration instead of 178); one kernel holds both there.
+// A block one barrier ahead writes the other half of the slots; it cannot be
+// two ahead.  Returns false if the wait ran out (ctrl->status is then
+// DS_TIMEOUT) or another block flagged an error; the caller must then stop
+// working on this team's solve.
 //
-// All blocks of the team must be co-resident (cooperative launch).  `sh` needs
-// 32 * NS doubles of shared memory.
-template <int NS>
-__device__ __forceinline__ bool team_reduce_impl(const Team& tm, const double (&mine)[NS], double (&out)[NS], double* sh) {
+// All blocks of the team must be co-resident (cooperative launch), and every
+// thread has called team_begin before the block barrier of the first
+// block_sum.  `sh` needs 32 * NS doubles of shared memory.  Inlined, and the
+// sums passed through copies: by reference to a call the sums' owner, a sink
+// with all its coefficients, lives in local memory, where every node reads them
+// again (FP32 BiCGStab at 2048^2 187 us per iteration, so 168; FP64 CG-NB at
+// 1024^2 61 and 51).
+template <int NS, bool BOTH>
+__device__ __forceinline__ bool team_reduce_impl(const Team& tm, const double (&mine)[NS], double (&out)[NS],
+                                                 double* sh) {
   static_assert(NS <= RED_MAX, "partial-sum slots");
-  __shared__ int s_ok;
+  __shared__ int s_ok;   // 0: gave up, 1: released, 2: the last block, which sums for all
   const int tid = threadIdx.x;
   Ctrl* ctrl = tm.ctrl;
   const unsigned epoch = team_epoch();
+  const bool every = !BOTH || NS == 1 || tm.size <= 400;
   double* slots = tm.partials + (size_t)(epoch & 1u) * RED_MAX * tm.size;
   if (tid == 0) {
 #pragma unroll
     for (int s = 0; s < NS; s++) slots[(size_t)tm.rank * NS + s] = mine[s];
-    red_release(&ctrl->count, 1u);
-    const unsigned target = (epoch + 1u) * (unsigned)tm.size;   // compared modulo 2^32
+    const unsigned full = (epoch + 1u) * (unsigned)tm.size;   // compared modulo 2^32
     int ok = 1;
-    unsigned long long t0 = 0;
-    unsigned spins = 0;
-    while ((int)(ld_acquire(&ctrl->count) - target) < 0) {
-      if (++spins > 64) {
-        __nanosleep(100);
-        if ((spins & 255) == 0) {
-          if (t0 == 0) t0 = global_ns();
-          if (ld_acquire_int(&ctrl->status) < 0) { ok = 0; break; }
-          if (global_ns() - t0 > ctrl->timeout_ns) {
-            atomicCAS(&ctrl->status, 0, (int)DS_TIMEOUT);
-            ok = 0;
-            break;
+    if (every) red_release(&ctrl->count, 1u);
+    else if (atom_acq_rel(&ctrl->count, 1u) + 1u == full) ok = 2;
+    if (ok == 1) {
+      const unsigned* word = every ? &ctrl->count : &ctrl->gen;
+      const unsigned target = every ? full : epoch + 1u;
+      unsigned long long t0 = 0;
+      unsigned spins = 0;
+      while ((int)(ld_acquire(word) - target) < 0) {
+        if (++spins > 64) {
+          __nanosleep(100);
+          if ((spins & 255) == 0) {
+            if (t0 == 0) t0 = global_ns();
+            if (ld_acquire_int(&ctrl->status) < 0) { ok = 0; break; }
+            if (global_ns() - t0 > ctrl->timeout_ns) {
+              atomicCAS(&ctrl->status, 0, (int)DS_TIMEOUT);
+              ok = 0;
+              break;
+            }
           }
         }
       }
@@ -273,8 +288,14 @@ __device__ __forceinline__ bool team_reduce_impl(const Team& tm, const double (&
     s_ok = ok;
   }
   __syncthreads();
-  if (!s_ok) return false;
+  const int ok = s_ok;
+  if (!ok) return false;
   if (tid == 0) team_epoch() = epoch + 1u;
+  if (!every && ok == 1) {
+#pragma unroll
+    for (int s = 0; s < NS; s++) out[s] = __ldcg(&ctrl->scal[s]);
+    return true;
+  }
 #pragma unroll
   for (int s = 0; s < NS; s++) out[s] = 0.0;
   for (int b = tid; b < tm.size; b += blockDim.x) {
@@ -282,34 +303,47 @@ __device__ __forceinline__ bool team_reduce_impl(const Team& tm, const double (&
     for (int s = 0; s < NS; s++) out[s] += __ldcg(&slots[(size_t)b * NS + s]);
   }
   block_sum<NS>(out, sh);
+  if (!every && tid == 0) {
+#pragma unroll
+    for (int s = 0; s < NS; s++) ctrl->scal[s] = out[s];
+    st_release(&ctrl->gen, epoch + 1u);
+  }
   return true;
 }
-
-// Called or inlined: inlined (InlineTeam), Jacobi and the FP64 neighbour-sum
-// kernels run faster (256^3 Jacobi 109 against 115 us per sweep, 250 x 187 x 141
-// 64 against 82, 128^2 BiCGStab 22.9 against 25.2); the other stencil passes
-// lose registers to it (FP32 CG on stored coefficients, one node per lane: 76
-// bytes of spills, 285 instead of 249 us per iteration).
-template <int NS>
-__device__ __noinline__ bool team_reduce(const Team& tm, const double (&mine)[NS], double (&out)[NS], double* sh) {
-  return team_reduce_impl<NS>(tm, mine, out, sh);
+template <int NS, bool BOTH>
+__device__ __forceinline__ bool team_reduce_copies(const Team tm, const double (&mine)[NS], double (&out)[NS],
+                                                   double* sh) {
+  double m[NS], r[NS];
+#pragma unroll
+  for (int s = 0; s < NS; s++) m[s] = mine[s];
+  const bool ok = team_reduce_impl<NS, BOTH>(tm, m, r, sh);
+#pragma unroll
+  for (int s = 0; s < NS; s++) out[s] = r[s];
+  return ok;
 }
-struct InlineTeam : Team {};
 template <int NS>
-__device__ __forceinline__ bool team_reduce(const InlineTeam& tm, const double (&mine)[NS], double (&out)[NS],
+__device__ __forceinline__ bool team_reduce(const Team& tm, const double (&mine)[NS], double (&out)[NS], double* sh) {
+  return team_reduce_copies<NS, false>(tm, mine, out, sh);
+}
+struct BiTeam : Team {};
+template <int NS>
+__device__ __forceinline__ bool team_reduce(const BiTeam& tm, const double (&mine)[NS], double (&out)[NS],
                                             double* sh) {
-  return team_reduce_impl<NS>(tm, mine, out, sh);
+  return team_reduce_copies<NS, true>(tm, mine, out, sh);
 }
 
-// The teams of a batch: the last block to arrive sums the partials in rank
-// order, publishes the sums and releases the others.  Six trips to L2 instead
-// of three, but fewer registers and loads in the batch kernels, which spill
-// already (48 systems of 16 to 24 nodes a side, 40 iterations: 4.10 ms against
-// 4.64 with team_reduce above; up to 128 a side: 27.1 against 27.7).
-struct BatchTeam : Team {};
+// LastTeam: the last block to arrive sums the partials in rank order, publishes
+// the sums and releases the others.  Six trips to L2 instead of three, but
+// fewer registers: for the batch kernels, which spill already (48 systems of 16
+// to 24 nodes a side, 40 iterations: 4.10 ms against 4.64 with team_reduce
+// above; up to 128 a side: 27.1 against 27.7), and for Gauss-Seidel, which has
+// a barrier per residual check and not per sweep (256^3, 20 pipelined sweeps:
+// 436 us each against 444; the 27-point form 4.27 ms against 4.50).  Its slots:
+// NS * size partials.
+struct LastTeam : Team {};
 
 template <int NS>
-__device__ bool team_reduce(const BatchTeam& tm, const double (&mine)[NS], double (&out)[NS], double* sh) {
+__device__ bool team_reduce(const LastTeam& tm, const double (&mine)[NS], double (&out)[NS], double* sh) {
   __shared__ int s_last;
   __shared__ int s_ok;
   Ctrl* ctrl = tm.ctrl;
@@ -382,6 +416,25 @@ __device__ __forceinline__ bool team_sync(const TM& tm, double* sh) {
   __syncthreads();
   double z[1] = {0.0}, o[1];
   return team_reduce<1>(tm, z, o, sh);
+}
+
+template <class TM = Team>
+__device__ __forceinline__ TM grid_team(Ctrl* ctrl, double* partials) {
+  TM t;
+  t.rank = blockIdx.x;
+  t.size = gridDim.x;
+  t.ctrl = ctrl;
+  t.partials = partials;
+  return t;
+}
+// Whole-grid forms of LastTeam (Gauss-Seidel).
+template <int NS>
+__device__ __forceinline__ bool grid_reduce(Ctrl* ctrl, double* partials, const double (&mine)[NS],
+                                            double (&out)[NS], double* sh) {
+  return team_reduce<NS>(grid_team<LastTeam>(ctrl, partials), mine, out, sh);
+}
+__device__ __forceinline__ bool grid_sync(Ctrl* ctrl, double* partials, double* sh) {
+  return team_sync(grid_team<LastTeam>(ctrl, partials), sh);
 }
 
 }  // namespace hs

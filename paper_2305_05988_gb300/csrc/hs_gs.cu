@@ -341,7 +341,12 @@ __global__ void __launch_bounds__(gs_threads<NDIM, W>()) k_gs(GsArgs<T> a) {
   double* sh = reinterpret_cast<double*>(smraw);
   const long long N = a.g.N;
 
-  const Team tm = grid_team(a.cm.ctrl, a.cm.partials);
+  // the large tiles of single and symmetric sweeps run faster with Team (96^3
+  // symmetric 931 us against 957, one 256^3 sweep 1789 against 1826), the small
+  // ones of pipelined batches with LastTeam (96^3 98 us per sweep against 104):
+  // the kernels' registers differ, barriers are few in either
+  using TM = std::conditional_t<W == 1, Team, LastTeam>;
+  if constexpr (W == 1) team_begin();
   double acc[1] = {0.0};
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
     T bv = a.b[i];
@@ -356,7 +361,7 @@ __global__ void __launch_bounds__(gs_threads<NDIM, W>()) k_gs(GsArgs<T> a) {
   unsigned long long cbase = 0;
   block_sum<1>(acc, sh);
   double bb[1];
-  if (!team_reduce<1>(tm, acc, bb, sh)) return;
+  if (!team_reduce<1>(grid_team<TM>(a.cm.ctrl, a.cm.partials), acc, bb, sh)) return;
   if (bb[0] == 0.0) {
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x)
       a.x[i] = T(0);
@@ -371,7 +376,7 @@ __global__ void __launch_bounds__(gs_threads<NDIM, W>()) k_gs(GsArgs<T> a) {
   int done = 0, status = DS_CONVERGED;
   double rel = -1.0;
   if (a.tol > 0.0) {
-    if (!gs_residual<T, OPK, NDIM>(a, tm, sh, bb[0], &rel)) return;
+    if (!gs_residual<T, OPK, NDIM, TM>(a, sh, bb[0], &rel)) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) a.cm.hist[0] = rel;
     if (!(rel > a.tol)) status = isfinite(rel) ? DS_CONVERGED : DS_NONFINITE;
     else status = DS_MAXIT;
@@ -383,7 +388,7 @@ __global__ void __launch_bounds__(gs_threads<NDIM, W>()) k_gs(GsArgs<T> a) {
         return;
       done += nb;
       if (a.tol > 0.0) {
-        if (!gs_residual<T, OPK, NDIM>(a, tm, sh, bb[0], &rel)) return;
+        if (!gs_residual<T, OPK, NDIM, TM>(a, sh, bb[0], &rel)) return;
         if (blockIdx.x == 0 && threadIdx.x == 0) {
           for (int q = done - nb + 1; q < done; q++) a.cm.hist[q] = nan("");  // not evaluated
           a.cm.hist[done] = rel;

@@ -47,11 +47,11 @@ struct GsArgs {
 // reduced over the grid.  Neighbours come straight from global memory (a
 // residual is formed once per check_every sweeps, so no tile staging; this
 // also frees the GS block from the tile engine's three-warp minimum).
-template <typename T, int OPK, int NDIM>
-__device__ bool gs_residual(const GsArgs<T>& a, const Team& tm, double* sh, double bb, double* rel) {
+template <typename T, int OPK, int NDIM, class TM>
+__device__ bool gs_residual(const GsArgs<T>& a, double* sh, double bb, double* rel) {
   const Geom& g = a.g;
   // blocks leave a batch at different times
-  if (!team_sync(tm, sh)) return false;
+  if (!team_sync(grid_team<TM>(a.cm.ctrl, a.cm.partials), sh)) return false;
   const T* bsrc = (OPK == OP_VARK) ? a.b : a.bD;
   const T* x = a.x;
   double acc[1] = {0.0};
@@ -75,7 +75,7 @@ __device__ bool gs_residual(const GsArgs<T>& a, const Team& tm, double* sh, doub
   }
   block_sum<1>(acc, sh);
   double rr[1];
-  if (!team_reduce<1>(tm, acc, rr, sh)) return false;
+  if (!team_reduce<1>(grid_team<TM>(a.cm.ctrl, a.cm.partials), acc, rr, sh)) return false;
   const double sc = (OPK == OP_VARK) ? 1.0 : a.dscale2;
   *rel = sqrt(rr[0] * sc / bb);
   return true;

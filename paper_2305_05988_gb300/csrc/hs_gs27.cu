@@ -220,10 +220,10 @@ __device__ __forceinline__ bool gs27_batch(const Gs27Args<T>& a, unsigned long l
 
 // Relative residual through the Jacobi form, reduced over the grid.
 template <typename T>
-__device__ bool gs27_residual(const Gs27Args<T>& a, const Team& tm, double* sh, double bb, double* rel) {
+__device__ bool gs27_residual(const Gs27Args<T>& a, double* sh, double bb, double* rel) {
   const Geom& g = a.g;
   // blocks finish a batch at different times: all sweeps must be complete
-  if (!team_sync(tm, sh)) return false;
+  if (!grid_sync(a.cm.ctrl, a.cm.partials, sh)) return false;
   double acc[1] = {0.0};
   for (long long idx = gtid(); idx < g.N; idx += gstride()) {
     const int i = (int)(idx % g.nx);
@@ -243,7 +243,7 @@ __device__ bool gs27_residual(const Gs27Args<T>& a, const Team& tm, double* sh, 
   }
   block_sum<1>(acc, sh);
   double rr[1];
-  if (!team_reduce<1>(tm, acc, rr, sh)) return false;
+  if (!grid_reduce<1>(a.cm.ctrl, a.cm.partials, acc, rr, sh)) return false;
   *rel = sqrt(rr[0] * a.dscale2 / bb);
   return true;
 }
@@ -256,7 +256,6 @@ __device__ bool gs27_residual(const Gs27Args<T>& a, const Team& tm, double* sh, 
 template <typename T, class Batch>
 __device__ __forceinline__ void gs27_solve(const Gs27Args<T>& a, double* sh, Batch&& batch) {
   const long long N = a.g.N;
-  const Team tm = grid_team(a.cm.ctrl, a.cm.partials);
   double acc[1] = {0.0};
   for (long long i = gtid(); i < N; i += gstride()) {
     const T bv = a.b[i];
@@ -265,7 +264,7 @@ __device__ __forceinline__ void gs27_solve(const Gs27Args<T>& a, double* sh, Bat
   }
   block_sum<1>(acc, sh);
   double bb[1];
-  if (!team_reduce<1>(tm, acc, bb, sh)) return;
+  if (!grid_reduce<1>(a.cm.ctrl, a.cm.partials, acc, bb, sh)) return;
   if (bb[0] == 0.0) {
     for (long long i = gtid(); i < N; i += gstride()) a.x[i] = T(0);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -279,7 +278,7 @@ __device__ __forceinline__ void gs27_solve(const Gs27Args<T>& a, double* sh, Bat
   int done = 0, status = DS_CONVERGED;
   double rel = -1.0;
   if (a.tol > 0.0) {
-    if (!gs27_residual(a, tm, sh, bb[0], &rel)) return;
+    if (!gs27_residual(a, sh, bb[0], &rel)) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) a.cm.hist[0] = rel;
     status = !(rel > a.tol) ? (isfinite(rel) ? DS_CONVERGED : DS_NONFINITE) : DS_MAXIT;
   }
@@ -296,7 +295,7 @@ __device__ __forceinline__ void gs27_solve(const Gs27Args<T>& a, double* sh, Bat
       }
       done += nb;
       if (a.tol > 0.0) {
-        if (!gs27_residual(a, tm, sh, bb[0], &rel)) return;
+        if (!gs27_residual(a, sh, bb[0], &rel)) return;
         if (blockIdx.x == 0 && threadIdx.x == 0) {
           for (int q = done - nb + 1; q < done; q++) a.cm.hist[q] = __longlong_as_double(0x7ff8000000000000LL);   // not evaluated (quiet NaN)
           a.cm.hist[done] = rel;

@@ -305,7 +305,6 @@ template <typename T, int OPK, bool VEC>
 __global__ void __launch_bounds__(32 * GSP_WARPS, HS_GSP_MINB) k_gsp(GsArgs<T> a, GspArgs G) {
   __shared__ double sh[32 * MAX_SCAL];
   const long long N = a.g.N;
-  const Team tm = grid_team(a.cm.ctrl, a.cm.partials);
   double acc[1] = {0.0};
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
     T bv = a.b[i];
@@ -318,7 +317,7 @@ __global__ void __launch_bounds__(32 * GSP_WARPS, HS_GSP_MINB) k_gsp(GsArgs<T> a
   unsigned gsweep = 0;
   block_sum<1>(acc, sh);
   double bb[1];
-  if (!team_reduce<1>(tm, acc, bb, sh)) return;
+  if (!grid_reduce<1>(a.cm.ctrl, a.cm.partials, acc, bb, sh)) return;
   if (bb[0] == 0.0) {
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x)
       a.x[i] = T(0);
@@ -333,7 +332,7 @@ __global__ void __launch_bounds__(32 * GSP_WARPS, HS_GSP_MINB) k_gsp(GsArgs<T> a
   int done = 0, status = DS_CONVERGED;
   double rel = -1.0;
   if (a.tol > 0.0) {
-    if (!gs_residual<T, OPK, 3>(a, tm, sh, bb[0], &rel)) return;
+    if (!gs_residual<T, OPK, 3, LastTeam>(a, sh, bb[0], &rel)) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) a.cm.hist[0] = rel;
     if (!(rel > a.tol)) status = isfinite(rel) ? DS_CONVERGED : DS_NONFINITE;
     else status = DS_MAXIT;
@@ -344,7 +343,7 @@ __global__ void __launch_bounds__(32 * GSP_WARPS, HS_GSP_MINB) k_gsp(GsArgs<T> a
       if (!gsp_batch<T, OPK, VEC>(a, G, a.mode == HS_GS_SYMMETRIC ? 2 * nb : nb, a.mode, gsweep)) return;
       done += nb;
       if (a.tol > 0.0) {
-        if (!gs_residual<T, OPK, 3>(a, tm, sh, bb[0], &rel)) return;
+        if (!gs_residual<T, OPK, 3, LastTeam>(a, sh, bb[0], &rel)) return;
         if (blockIdx.x == 0 && threadIdx.x == 0) {
           for (int q = done - nb + 1; q < done; q++) a.cm.hist[q] = nan("");  // not evaluated
           a.cm.hist[done] = rel;

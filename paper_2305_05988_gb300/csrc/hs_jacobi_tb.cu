@@ -152,6 +152,7 @@ __global__ void __launch_bounds__(tb_threads<S>()) k_jacobi_tb(JacTbArgs<T> a) {
   __shared__ double sh[32 * MAX_SCAL];
   T* sm = reinterpret_cast<T*>(smraw);
   const long long N = a.g.N;
+  team_begin();
   const Team tm = grid_team(a.cm.ctrl, a.cm.partials);
   double acc[1] = {0.0};
   for (long long i = gtid(); i < N; i += gstride()) {

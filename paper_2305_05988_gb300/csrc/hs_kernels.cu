@@ -204,7 +204,8 @@ __global__ void __launch_bounds__(512) __maxnreg__((jac_maxnreg<T, OPK, NDIM, CX
   T* sm = reinterpret_cast<T*>(smraw);
   const long long N = a.g.N;
 
-  const InlineTeam tm = grid_team<InlineTeam>(a.cm.ctrl, a.cm.partials);
+  team_begin();
+  const Team tm = grid_team(a.cm.ctrl, a.cm.partials);
   double acc[1] = {0.0};
   for (long long i = gtid(); i < N; i += gstride()) {
     T bv = a.b[i];
@@ -316,8 +317,8 @@ template <typename T, int OPK, int NDIM, int CX>
 __global__ void __launch_bounds__(512) __maxnreg__((cg_maxnreg<T, OPK, NDIM, CX>())) k_cg(CgArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ double sh[32 * MAX_SCAL];
-  using TM = std::conditional_t<fx_op(OPK), InlineTeam, Team>;
-  const TM tm = grid_team<TM>(a.cm.ctrl, a.cm.partials);
+  const Team tm = grid_team(a.cm.ctrl, a.cm.partials);
+  team_begin();
   constexpr bool xdefer = HS_CG_XDEFER && sizeof(T) == 8 && OPK != OP_VARK;
   team_finish(tm, cg_body<T, OPK, NDIM, CX, xdefer>(a, tm, reinterpret_cast<T*>(smraw), sh));
 }
@@ -326,8 +327,8 @@ template <typename T, int OPK, int NDIM>
 __global__ void __launch_bounds__(512) __maxnreg__((bi_maxnreg<T, OPK, NDIM>())) k_bicgstab(BiArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ double sh[32 * MAX_SCAL];
-  using TM = std::conditional_t<fx_op(OPK), InlineTeam, Team>;
-  const TM tm = grid_team<TM>(a.cm.ctrl, a.cm.partials);
+  const BiTeam tm = grid_team<BiTeam>(a.cm.ctrl, a.cm.partials);
+  team_begin();
   team_finish(tm, bicgstab_body<T, OPK, NDIM>(a, tm, reinterpret_cast<T*>(smraw), sh));
 }
 
@@ -338,6 +339,7 @@ __global__ void __launch_bounds__(512) __maxnreg__((bi_maxnreg<T, OPK, NDIM>()))
 __global__ void k_init_ctrl(Ctrl* c, unsigned long long timeout_ns) {
   if (threadIdx.x == 0) {
     c->count = 0;
+    c->gen = 0;
     c->status = 0;
     c->iters = 0;
     c->restarts = 0;
