@@ -255,6 +255,22 @@ struct ApDotSink {
   }
 };
 
+// Block-uniform scalars that an iteration carries from pass to pass, in the
+// part of the reduction scratch that block_sum<RED_MAX> leaves free: held in
+// registers they are spilled inside the marches (FP32 CG on stored
+// coefficients, one node per lane, 250 x 187 x 141: 169 us per iteration, 152
+// so).  Set by every block's thread 0 behind a reduction; a reduction lies
+// between a set and the next get of a slot, and between a get and the next set.
+struct Keep {
+  volatile double* s;
+  __device__ __forceinline__ explicit Keep(double* sh) : s(sh + 32 * RED_MAX) {}
+  __device__ __forceinline__ double get(int q) const { return s[q]; }
+  __device__ __forceinline__ void set(int q, double v) const {
+    if (threadIdx.x == 0) s[q] = v;
+  }
+};
+static_assert(MAX_SCAL > RED_MAX, "the reduction scratch holds the kept scalars");
+
 // The CG iteration run by one team of blocks (the whole grid for a standalone
 // solve, a subset of blocks in the batched solver).
 // XDEFER: the x update of iteration k runs in pass 1 of iteration k+1
@@ -276,19 +292,23 @@ __device__ BodyOut cg_body(const CgArgs<T>& a, const TM& tm, T* sm, double* sh) 
   block_sum<2>(rsink.acc, sh);
   double s2[2];
   if (!team_reduce<2>(tm, rsink.acc, s2, sh)) return BodyOut{DS_TIMEOUT, 0, -1.0, 0, false};
-  double rr = s2[0];
   const double bb = s2[1];
   if (bb == 0.0) {
     for (long long i = tm.tid(); i < N; i += tm.stride()) a.x[i] = T(0);
     if (tm.lead() && a.cm.hist) a.cm.hist[0] = 0.0;
     return BodyOut{DS_CONVERGED, 0, 0.0, 0, true};
   }
-  double rel = sqrt(rr / bb);
+  double rel = sqrt(s2[0] / bb);
   if (tm.lead() && a.cm.hist) a.cm.hist[0] = rel;
   if (rel <= a.tol || a.maxit == 0) {
     return BodyOut{rel <= a.tol ? DS_CONVERGED : DS_MAXIT, 0, rel, 0, true};
   }
 
+  const Keep keep(sh);
+  enum { RR = 0, BB = 2, REL = 3 };   // r.r of iteration k in slot k & 1
+  keep.set(RR, s2[0]);
+  keep.set(BB, bb);
+  keep.set(REL, rel);
   double beta = 0.0, alpha_prev = 0.0;
   bool first = true;
   int it = 0, status = DS_MAXIT;
@@ -310,12 +330,12 @@ __device__ BodyOut cg_body(const CgArgs<T>& a, const TM& tm, T* sm, double* sh) 
       acc0[0] = sink.acc[0];
     }
     block_sum<1>(acc0, sh);
-    if (!team_reduce<1>(tm, acc0, pw, sh)) return BodyOut{DS_TIMEOUT, it, rel, 0, false};
+    if (!team_reduce<1>(tm, acc0, pw, sh)) return BodyOut{DS_TIMEOUT, it, keep.get(REL), 0, false};
     if (!(pw[0] > 0.0) || !finite_d(pw[0])) {
       status = finite_d(pw[0]) ? DS_BREAKDOWN : DS_NONFINITE;
-      return BodyOut{status, it, rel, 0, true};   // x holds x_{it-1} in both forms
+      return BodyOut{status, it, keep.get(REL), 0, true};   // x holds x_{it-1} in both forms
     }
-    const double ar = rr / pw[0];           // multiplies w = A p / sigma
+    const double ar = keep.get(RR + ((it - 1) & 1)) / pw[0];           // multiplies w = A p / sigma
     const T tar = (T)ar;
     double acc1[1] = {0.0};
     if constexpr (XDEFER) {
@@ -410,9 +430,9 @@ __device__ BodyOut cg_body(const CgArgs<T>& a, const TM& tm, T* sm, double* sh) 
     }
     block_sum<1>(acc1, sh);
     double rn[1];
-    if (!team_reduce<1>(tm, acc1, rn, sh)) return BodyOut{DS_TIMEOUT, it, rel, 0, false};
+    if (!team_reduce<1>(tm, acc1, rn, sh)) return BodyOut{DS_TIMEOUT, it, keep.get(REL), 0, false};
     alpha_prev = ar;
-    rel = sqrt(rn[0] / bb);
+    rel = sqrt(rn[0] / keep.get(BB));
     if (tm.lead() && a.cm.hist) a.cm.hist[it] = rel;
     if (!finite_d(rel)) {
       status = DS_NONFINITE;
@@ -422,8 +442,9 @@ __device__ BodyOut cg_body(const CgArgs<T>& a, const TM& tm, T* sm, double* sh) 
       status = DS_CONVERGED;
       break;
     }
-    beta = rn[0] / rr;
-    rr = rn[0];
+    beta = rn[0] / keep.get(RR + ((it - 1) & 1));
+    keep.set(RR + (it & 1), rn[0]);
+    keep.set(REL, rel);
     first = false;
   }
   // the last step of x, x += alpha p (same element -> thread map as the
@@ -611,8 +632,7 @@ __device__ BodyOut bicgstab_body(const BiArgs<T>& a, const TM& tm, T* sm, double
   block_sum<2>(rsink.acc, sh);
   double s2[2];
   if (!team_reduce<2>(tm, rsink.acc, s2, sh)) return BodyOut{DS_TIMEOUT, 0, -1.0, 0, false};
-  double brr = s2[0];
-  const double bb = s2[1];
+  const double brr = s2[0], bb = s2[1];
   if (bb == 0.0) {
     for (long long i = tm.tid(); i < N; i += tm.stride()) a.x[i] = T(0);
     if (tm.lead() && a.cm.hist) a.cm.hist[0] = 0.0;
@@ -624,10 +644,14 @@ __device__ BodyOut bicgstab_body(const BiArgs<T>& a, const TM& tm, T* sm, double
     return BodyOut{rel <= a.tol ? DS_CONVERGED : DS_MAXIT, 0, rel, 0, true};
   }
 
-  double alpha_n = sqrt(brr);   // r . r' with r' = r / ||r||
+  const Keep keep(sh);
+  enum { ALPHA_N, BB, REL, ALPHA, ALPHA_D };
+  keep.set(ALPHA_N, sqrt(brr));   // r . r' with r' = r / ||r||
+  keep.set(BB, bb);
+  keep.set(REL, rel);
   double inv_rn = 1.0 / sqrt(brr);
   if (tm.lead() && a.trace) {
-    a.trace[0] = alpha_n;
+    a.trace[0] = sqrt(brr);
     a.trace[1] = 0.0;
   }
   bool restart = true;          // p = r and r' = r/||r|| in the next pass 1
@@ -658,27 +682,31 @@ __device__ BodyOut bicgstab_body(const BiArgs<T>& a, const TM& tm, T* sm, double
         acc1[0] = sink.acc[0];
       }
       block_sum<1>(acc1, sh);
-      if (!team_reduce<1>(tm, acc1, ad, sh)) return BodyOut{DS_TIMEOUT, it, rel, restarts, false};
+      if (!team_reduce<1>(tm, acc1, ad, sh)) return BodyOut{DS_TIMEOUT, it, keep.get(REL), restarts, false};
     }
+    rel = keep.get(REL);
     const double alpha_d = a.sigma * ad[0];
     if (alpha_d == 0.0 || !finite_d(alpha_d)) {
       status = finite_d(alpha_d) ? DS_BREAKDOWN : DS_NONFINITE;
       break;
     }
-    const double alpha = alpha_n / alpha_d;
     // ---- pass 2
     double st3[3];
     {
+      const double alpha = keep.get(ALPHA_N) / alpha_d;
+      keep.set(ALPHA, alpha);
+      keep.set(ALPHA_D, alpha_d);
       BiSSrc<T> src{a.r, vnew, a.s, (T)(alpha * a.sigma)};
       BiTSink<T, OPK, NDIM> sink{a.cf, a.g, a.t, {0.0, 0.0, 0.0}};
       for (int item = tm.rank; item < a.tl.items(); item += tm.size)
         zmarch_item<T, NDIM, CX>(a.g, a.tl, item, sm, src, sink);
       block_sum<3>(sink.acc, sh);
-      if (!team_reduce<3>(tm, sink.acc, st3, sh)) return BodyOut{DS_TIMEOUT, it, rel, restarts, false};
+      if (!team_reduce<3>(tm, sink.acc, st3, sh)) return BodyOut{DS_TIMEOUT, it, keep.get(REL), restarts, false};
     }
-    const double srel = sqrt(st3[0] / bb);
+    rel = keep.get(REL);
+    const double srel = sqrt(st3[0] / keep.get(BB));
     if (!a.paper_order && srel <= a.tol) {
-      const T ta = (T)alpha;
+      const T ta = (T)keep.get(ALPHA);
       for (long long i = tm.tid(); i < N; i += st) a.x[i] = fma(ta, ldcg(pnew + i), ldcg(a.x + i));
       if (tm.lead() && a.cm.hist) a.cm.hist[it] = srel;
       rel = srel;
@@ -695,7 +723,7 @@ __device__ BodyOut bicgstab_body(const BiArgs<T>& a, const TM& tm, T* sm, double
       status = DS_BREAKDOWN;
       break;
     }
-    const T ta = (T)alpha, tom = (T)omega, toms = (T)(omega * a.sigma);
+    const T ta = (T)keep.get(ALPHA), tom = (T)omega, toms = (T)(omega * a.sigma);
     if (a.paper_order && rel <= a.tol) {
       // Algorithm 2's order: the test on the residual of x_j comes after
       // omega_j, and the loop ends with x = x_j + alpha_j p_j + omega_j s_j
@@ -742,8 +770,9 @@ __device__ BodyOut bicgstab_body(const BiArgs<T>& a, const TM& tm, T* sm, double
     }
     block_sum<2>(acc4, sh);
     double rn2[2];
-    if (!team_reduce<2>(tm, acc4, rn2, sh)) return BodyOut{DS_TIMEOUT, it, rel, restarts, false};
-    rel = sqrt(rn2[1] / bb);
+    if (!team_reduce<2>(tm, acc4, rn2, sh)) return BodyOut{DS_TIMEOUT, it, keep.get(REL), restarts, false};
+    rel = sqrt(rn2[1] / keep.get(BB));
+    keep.set(REL, rel);
     if (tm.lead() && a.cm.hist) a.cm.hist[it] = rel;
     if (tm.lead() && a.trace) {
       a.trace[2 * it] = rn2[0];
@@ -759,13 +788,13 @@ __device__ BodyOut bicgstab_body(const BiArgs<T>& a, const TM& tm, T* sm, double
     }
     if (a.reps > 0.0 && sqrt(fabs(rn2[0])) < a.reps) {
       restart = true;
-      alpha_n = sqrt(rn2[1]);
+      keep.set(ALPHA_N, sqrt(rn2[1]));
       inv_rn = 1.0 / sqrt(rn2[1]);
       restarts++;
     } else {
       restart = false;
-      beta = rn2[0] / (alpha_d * omega);
-      alpha_n = rn2[0];
+      beta = rn2[0] / (keep.get(ALPHA_D) * omega);
+      keep.set(ALPHA_N, rn2[0]);
     }
     if (tm.lead() && a.trace && restart) a.trace[2 * it + 1] = 1.0;
   }
