@@ -204,7 +204,7 @@ static int batch_kind(const hs_op* A, int solver) {
   return d3 ? BK_BI_VARK3 : BK_BI_VARK2;
 }
 
-static size_t batch_smem() { return slab_bytes<double, OP_SYM>(BATCH_BY, BATCH_CX); }
+static size_t batch_smem() { return slab_bytes<double, OP_SYM, 3>(BATCH_BY, BATCH_CX); }
 
 static int cx_of(int) { return BATCH_CX; }
 

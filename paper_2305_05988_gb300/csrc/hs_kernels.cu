@@ -41,8 +41,9 @@ __global__ void __launch_bounds__(512) k_residual(Geom g, Tiling tl, Coef<T> cf,
   LoadSrc<T, false> src{x};
   ResidualSink<T, OPK, NDIM> sink{cf, g, sigma, b, r, {0.0, 0.0}};
   for (int item = blockIdx.x; item < tl.items(); item += gridDim.x) zmarch_item<T, NDIM, cx_st<OPK>()>(g, tl, item, sm, src, sink);
+  if (!partials) return;
   block_sum<2>(sink.acc, sh);
-  if (partials && threadIdx.x == 0) {
+  if (threadIdx.x == 0) {
     partials[2 * blockIdx.x] = sink.acc[0];
     partials[2 * blockIdx.x + 1] = sink.acc[1];
   }
@@ -612,10 +613,10 @@ static hs_status spmv_vark_direct(const hs_op* A, const void* x, void* y, cudaSt
   double ih[3];
   for (int d = 0; d < 3; d++) ih[d] = d < A->ndim ? 1.0 / (A->h[d] * A->h[d]) : 0.0;
   if (A->kdt == HS_F64)
-    k_spmv_vark_direct<T, double, NDIM><<<tl.items(), 32 * by, slab_bytes<T, OP_VARK>(by, CX_ST), st>>>(
+    k_spmv_vark_direct<T, double, NDIM><<<tl.items(), 32 * by, slab_bytes<T, OP_VARK, NDIM>(by, CX_ST), st>>>(
         g, tl, (const double*)A->k, ih[0], ih[1], ih[2], (const T*)x, (T*)y);
   else
-    k_spmv_vark_direct<T, float, NDIM><<<tl.items(), 32 * by, slab_bytes<T, OP_VARK>(by, CX_ST), st>>>(
+    k_spmv_vark_direct<T, float, NDIM><<<tl.items(), 32 * by, slab_bytes<T, OP_VARK, NDIM>(by, CX_ST), st>>>(
         g, tl, (const float*)A->k, ih[0], ih[1], ih[2], (const T*)x, (T*)y);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? HS_OK : cuda_fail(e, "spmv launch");
@@ -632,7 +633,7 @@ hs_status run_spmv(const hs_op* A, hs_dtype dt, const void* x, void* y, cudaStre
     Coef<T> cf = op_coef<T>(A, nullptr, nullptr, nullptr, nullptr, &sigma);
     int by = rows_per_tile(g);
     Tiling tl = choose_tiling(g, by, 0, false, 0, cx_st<OPK>());
-    k_spmv<T, OPK, NDIM><<<tl.items(), 32 * by, slab_bytes<T, OPK>(by, cx_st<OPK>()), st>>>(g, tl, cf, (T)sigma, (const T*)x, (T*)y);
+    k_spmv<T, OPK, NDIM><<<tl.items(), 32 * by, slab_bytes<T, OPK, NDIM>(by, cx_st<OPK>()), st>>>(g, tl, cf, (T)sigma, (const T*)x, (T*)y);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? hs_dbg_take(st) : cuda_fail(e, "spmv launch");
   });
@@ -661,7 +662,7 @@ hs_status run_residual_plain(const hs_op* A, hs_dtype dt, const void* b, const v
     Coef<T> cf = op_coef<T>(A, nullptr, nullptr, nullptr, nullptr, &sigma);
     int by = rows_per_tile(g);
     Tiling tl = choose_tiling(g, by, 0, false, 0, cx_st<OPK>());
-    k_residual<T, OPK, NDIM><<<tl.items(), 32 * by, slab_bytes<T, OPK>(by, cx_st<OPK>()), st>>>(g, tl, cf, (T)sigma, (const T*)b,
+    k_residual<T, OPK, NDIM><<<tl.items(), 32 * by, slab_bytes<T, OPK, NDIM>(by, cx_st<OPK>()), st>>>(g, tl, cf, (T)sigma, (const T*)b,
                                                                                (const T*)x, (T*)r, nullptr);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? hs_dbg_take(st) : cuda_fail(e, "residual launch");
@@ -684,7 +685,10 @@ static hs_status residual_norms(const hs_op* A, hs_dtype dt, const void* D, cons
     constexpr int cx = cx_st<OPK>();   // must match the kernel's columns per lane
     Tiling tl = choose_tiling(g, by, 0, false, 0, cx);
     int grid = std::min(tl.items(), MAX_BLOCKS * MAX_SCAL / 2);
-    k_residual<T, OPK, NDIM><<<grid, 32 * by, slab_bytes<T, OPK>(by, cx), st>>>(g, tl, cf, (T)sigma, (const T*)b,
+    // a 2-D tile has 256 nodes: blocks take several of them, or the sums over
+    // the block (80 FP64 additions of a warp) cost more than the stencil
+    if (NDIM == 2) grid = std::min(grid, 8 * sm_count());
+    k_residual<T, OPK, NDIM><<<grid, 32 * by, slab_bytes<T, OPK, NDIM>(by, cx), st>>>(g, tl, cf, (T)sigma, (const T*)b,
                                                                         (const T*)x, (T*)r, partials_dev);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "residual launch");
@@ -903,7 +907,7 @@ hs_status run_jacobi(const SolveArgs& sa, hs_result* res, double* hist) {
     if (!quad) {
       const int by = rows_for(g, sa.o);
       constexpr int cx = cx_jac<T, OPK>();
-      const size_t smem = slab_bytes<T, OPK>(by, cx);
+      const size_t smem = slab_bytes<T, OPK, NDIM>(by, cx);
       s = a.fuse ? launch(k_jacobi<T, OPK, NDIM, true, cx>, 32 * by, by, cx, smem)
                  : launch(k_jacobi<T, OPK, NDIM, false, cx>, 32 * by, by, cx, smem);
     }
@@ -952,7 +956,7 @@ static hs_status cg_core(const hs_op* A, const Coef<T>& cf, double sigma, const 
   }
   const int by = rows_for(a.g, o);
   constexpr int cx = cx_cg<T, OPK>();
-  return launch(k_cg<T, OPK, NDIM, cx>, 32 * by, by, cx, slab_bytes<T, OPK>(by, cx, 2, 1));
+  return launch(k_cg<T, OPK, NDIM, cx>, 32 * by, by, cx, slab_bytes<T, OPK, NDIM>(by, cx, 2, 1));
 }
 
 template <typename T, int OPK, int NDIM>
@@ -982,7 +986,7 @@ static hs_status bicgstab_core(const hs_op* A, const Coef<T>& cf, double sigma, 
   hs_status s = init_ctrl(cm, o, st);
   if (s != HS_OK) return s;
   int by = rows_for(a.g, o);
-  size_t smem = slab_bytes<T, OPK>(by, CX_BI, 3, 1);
+  size_t smem = slab_bytes<T, OPK, NDIM>(by, CX_BI, 3, 1);
   int grid = 0;
   s = plan_persistent(k_bicgstab<T, OPK, NDIM>, 32 * by, smem, a.g, by, true, &grid, &a.tl, o, CX_BI);
   if (s != HS_OK) return s;

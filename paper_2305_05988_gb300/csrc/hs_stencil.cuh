@@ -50,12 +50,14 @@ __device__ __forceinline__ void decode_item(const Tiling& t, const Geom& g, int 
   z1 = min(g.nz, z0 + t.lz);
 }
 
-// Bytes of shared memory of the engine for
-// `by` rows; na, nb: staged operands of the source and the sink (fx_op).
-template <typename T, int OPK>
+// Bytes of shared memory of the engine for `by` rows; na, nb: staged operands
+// of the source and the sink (fx_op, 3-D: a 2-D tile has no next plane to
+// stage, and a ring it does not use would only take from the L1 cache).
+template <typename T, int OPK, int NDIM>
 inline size_t slab_bytes(int by, int cx, int na = 1, int nb = 1) {
   const size_t pl = (size_t)(by + 2) * (BX * cx + 2);
   if (!fx_op(OPK)) return 2 * pl * sizeof(T);
+  if (NDIM == 2) return 12 * pl;
   return 24 * pl + 8 * (size_t)FX_NS * (na * (32 * by + 96) + nb * 32 * by);
 }
 
