@@ -168,8 +168,10 @@ struct JacobiSink {
   }
 };
 
-// Register caps of the neighbour-sum engine's 3-D kernels (A/B at 256^3):
-// Jacobi 64 (107 us per sweep; 48: 125, 56: 111, 80: 110), CG 80 (241 us per
+// Register caps of the neighbour-sum engine's kernels (A/B at 256^3; CG and
+// BiCGStab in 3-D):
+// Jacobi 64 (107 us per sweep; 48: 125, 56: 111, 80: 110; 2-D too: upwind
+// 2048^2 60.6 us without a cap, 53; with a residual 3000 x 2000 147 and 96), CG 80 (241 us per
 // iteration; 56: 278, 64: 258, 72: 250, 96: 283), BiCGStab 80 (527; 64: 642,
 // 96: 570, 128: 552).
 #ifndef HS_JAC_ISO_MAXNREG
@@ -193,7 +195,7 @@ struct JacobiSink {
 template <typename T, int OPK, int NDIM, int CX>
 constexpr int jac_maxnreg() {
   if (CX == CX_QUAD) return HS_JACQ_MAXNREG;
-  if (fx_op(OPK)) return NDIM == 3 ? HS_JAC_ISO_MAXNREG : 128;
+  if (fx_op(OPK)) return HS_JAC_ISO_MAXNREG;
   if (OPK == OP_VARK) return sizeof(T) == 8 ? 80 : 128;   // FP64: three blocks per SM (230 us a sweep; two: 249)
   return sizeof(T) == 4 ? 64 : 128;                       // FP32: four
 }
@@ -844,9 +846,22 @@ hs_status finish_solve_pub(const SolveArgs& sa, const Common& cm, const void* D,
 }
 
 // ---- Jacobi -----------------------------------------------------------------
+constexpr int64_t JAC_2D_WEIGHTED_MAX = 7 << 19;   // nodes: three vectors of 29 MB
+
 hs_status run_jacobi(const SolveArgs& sa, hs_result* res, double* hist) {
   if (jacobi_tb_applies(sa)) return run_jacobi_tb(sa, res, hist);
-  return dispatch(sa.dtype, kernel_op(sa.A, sa.dtype), sa.A->ndim, [&](auto tag) -> hs_status {
+  int opk = kernel_op(sa.A, sa.dtype);
+  // 2-D tiles of the neighbour-sum engine have nothing in flight but their own
+  // loads: with weighted sums on grids whose three vectors leave the L2 cache a
+  // plain sweep is faster in the general form (us, general / weighted: upwind
+  // 1448^2 32.1 / 30.0, 1800^2 42.5 / 42.2, 2048^2 48.5 / 52.9, 2300^2 65.4 /
+  // 72.0; Laplacian 2048 x 1400 37.9 / 35.9, 3000 x 2000 73.0 / 76.8).  Equal
+  // couplings (2300^2 65.9 / 64.2) and sweeps with a residual (3000 x 2000 114 /
+  // 96) stay.
+  if ((opk == OP_WSYM || opk == OP_WNON) && sa.A->ndim == 2 && !(sa.tol > 0.0) &&
+      sa.A->n[0] * sa.A->n[1] > JAC_2D_WEIGHTED_MAX)
+    opk = opkind_of(sa.A);
+  return dispatch(sa.dtype, opk, sa.A->ndim, [&](auto tag) -> hs_status {
     using Tg = decltype(tag);
     using T = typename Tg::T;
     constexpr int OPK = Tg::OPK, NDIM = Tg::NDIM;
