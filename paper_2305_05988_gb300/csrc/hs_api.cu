@@ -330,6 +330,7 @@ static hs_status make_op(const hs_grid* g, int kind, const double* beta, const v
   }
   A->k = k;
   A->kdt = kdt;
+  set_op64(A);
   *out = A;
   return HS_OK;
 }

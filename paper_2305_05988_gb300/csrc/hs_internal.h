@@ -26,6 +26,8 @@ struct hs_op {
   double beta[3];
   const void* k;      // diffusion: borrowed device pointer
   int kdt;            // hs_dtype of k
+  int op64;           // OpKind the FP64 kernels are compiled for
+  hs::FxW fx;         // its weights (fx_op)
 };
 
 namespace hs {
@@ -100,21 +102,26 @@ ConstRow const_row(const hs_op* A);
 // they lie more than a factor of 64 apart.
 bool fx_weights(const hs_op* A, FxW* W);
 
-// The operator kind a kernel is compiled for.  FP64 operators in 2-D and 3-D
-// take the neighbour sum on the integer pipes where the couplings lie within
+// Fills in A->op64 and A->fx when an operator is created (a small SpMV takes
+// 5 us with its launch, the weights' twelve divisions 0.1).  FP64 operators in 2-D and
+// 3-D take the neighbour sum on the integer pipes where the couplings lie within
 // a factor of 64 (grid spacings within 8, cell Peclet numbers to 31).  The
 // error of the sums does not depend on the factor (fx_neighbours); up to there
 // they are tested against extended precision and timed.
-inline int kernel_op(const hs_op* A, hs_dtype dt) {
-  const int opk = opkind_of(A);
-  if ((opk != OP_SYM && opk != OP_NONSYM) || dt != HS_F64 || A->ndim < 2) return opk;
-  FxW W;
-  if (!fx_weights(A, &W)) return opk;
-  if (opk == OP_NONSYM) return OP_WNON;
+inline void set_op64(hs_op* A) {
+  A->op64 = opkind_of(A);
+  if ((A->op64 != OP_SYM && A->op64 != OP_NONSYM) || A->ndim < 2 || !fx_weights(A, &A->fx)) return;
+  if (A->op64 == OP_NONSYM) {
+    A->op64 = OP_WNON;
+    return;
+  }
+  A->op64 = OP_ISO;
   for (int q = 0; q < 2 * A->ndim; q++)
-    if (W.w[q] != 1.0) return OP_WSYM;
-  return OP_ISO;
+    if (A->fx.w[q] != 1.0) A->op64 = OP_WSYM;
 }
+
+// The operator kind a kernel is compiled for.
+inline int kernel_op(const hs_op* A, hs_dtype dt) { return dt == HS_F64 ? A->op64 : opkind_of(A); }
 
 // Chooses a tiling (rows per tile, z chunk length) for `grid` persistent
 // blocks sharing `sms` SMs (0: a team of a batch), or for a one-item-per-block

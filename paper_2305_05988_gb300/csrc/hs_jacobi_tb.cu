@@ -209,7 +209,7 @@ static hs_status jacobi_tb_t(const SolveArgs& sa, hs_result* res, double* hist) 
     a.cf.zl = (T)(-r.zl / r.d);
     a.cf.zu = (T)(-r.zu / r.d);
     a.invd = (T)(1.0 / r.d);
-    if constexpr (std::is_same<T, double>::value) fx_weights(A, &a.cf.fx);
+    if constexpr (std::is_same<T, double>::value) a.cf.fx = A->fx;
   }
   a.g = g;
   a.b = (const T*)sa.b;

@@ -474,7 +474,7 @@ static Coef<T> jacobi_coef(const hs_op* A, T* invd, double* d2) {
   cf.zu = (T)(-c.zu / c.d);
   *invd = (T)(1.0 / c.d);
   *d2 = c.d * c.d;
-  if constexpr (std::is_same<T, double>::value) fx_weights(A, &cf.fx);
+  if constexpr (std::is_same<T, double>::value) cf.fx = A->fx;
   return cf;
 }
 

@@ -821,7 +821,7 @@ inline Coef<T> scaled_coef(const hs_op* A, double* sigma) {
   cf.zu = (T)(c.zu / s);
   // 27-point: A x = 27 x - (box - x) = 28 x - box (s = 1)
   if (A->kind == KIND_HPCG27) cf.d = (T)(c.d + 1.0);
-  if constexpr (std::is_same<T, double>::value) fx_weights(A, &cf.fx);
+  if constexpr (std::is_same<T, double>::value) cf.fx = A->fx;
   return cf;
 }
 
