@@ -825,6 +825,9 @@ inline Coef<T> scaled_coef(const hs_op* A, double* sigma) {
   return cf;
 }
 
+// Whether hs_opts.tile_rows is a choice; other values mean the heuristics.
+inline bool rows_chosen(const hs_opts& o) { return o.tile_rows >= 4 && o.tile_rows <= 16; }
+
 // Whether a solve takes the FP32 engine with four nodes per lane: x-lines of
 // whole quads (every vector is 16-byte aligned) that fill at least three
 // quarters of its 64-node tiles, rows per tile not chosen by the caller, and
@@ -833,7 +836,7 @@ inline Coef<T> scaled_coef(const hs_op* A, double* sigma) {
 // 192^3 101 / 79.9; Jacobi 64^3 6.2 / 6.1, 128^3 12.5 / 10.6, 192^3 28.4 / 19.1.
 inline bool quad_applies(const Geom& g, const hs_opts& o) {
   const int wide = (g.nx + QTW - 1) / QTW * QTW;
-  return g.nx % 4 == 0 && 4 * g.nx >= 3 * wide && o.tile_rows == 0 && g.nz > 1 && g.N >= (1 << 17);
+  return g.nx % 4 == 0 && 4 * g.nx >= 3 * wide && !rows_chosen(o) && g.nz > 1 && g.N >= (1 << 17);
 }
 
 inline int rows_per_tile(const Geom& g) {
@@ -845,7 +848,7 @@ inline int rows_per_tile(const Geom& g) {
 // Rows per tile: the caller's choice (hs_opts.tile_rows, 4 to 16) or the
 // heuristic above.
 inline int rows_for(const Geom& g, const hs_opts& o) {
-  if (o.tile_rows >= 4 && o.tile_rows <= 16) return o.tile_rows;
+  if (rows_chosen(o)) return o.tile_rows;
   return rows_per_tile(g);
 }
 
