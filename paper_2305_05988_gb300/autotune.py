@@ -1,7 +1,9 @@
 """Tile autotuner for the stencil solvers.
 
 The stencil tile engine has two shape parameters: rows of 32 nodes per tile
-(= warps per block, 4 / 8 / 16) and z planes per work item.  Their best values
+(= warps per block, 4 / 8 / 16) and z planes per work item.  0 rows, the
+library's own choice, is a candidate where that may be another engine: FP32
+Jacobi and CG in 3-D, four nodes per lane.  Their best values
 depend on the grid size, the dimension, the operator, the solver and the GPU.
 This module times short fixed-iteration solves (tol = 0, so every candidate
 does exactly the same arithmetic work) for each candidate shape with CUDA
@@ -12,6 +14,7 @@ events, keeps the fastest, and caches the winner in a JSON file keyed by
 where the size bucket is the grid's largest side rounded to a power of two and
 `team` is "grid" (standalone solve on every co-resident block) or "1" (a
 single block, the condition of a small system in the batched solver's queue).
+Entries carry the engines' version; those of another version are tuned again.
 
 Cache file: $HSOLVE_TUNE_CACHE, else ~/.cache/hsolve/tune.json.
 """
@@ -31,6 +34,7 @@ from .solvers import Operator, bicgstab, cg, jacobi
 
 _LOCK = threading.Lock()
 
+ENGINE = 2   # version of the kernels that the entries were timed with
 ROW_CANDIDATES = (4, 8, 16)
 PLANE_CANDIDATES = (0, 8, 16, 32, 64)
 
@@ -66,6 +70,18 @@ def save_cache(cache: Dict[str, dict], path: Optional[str] = None) -> None:
     with open(tmp, "w") as f:
         json.dump(cache, f, indent=1, sort_keys=True)
     os.replace(tmp, path)
+
+
+def row_candidates(shape: Sequence[int], solver: str, dtype, team: str) -> tuple:
+    """Rows per tile worth timing; 0 leaves the choice to the library."""
+    if team != "grid":
+        return (8,)
+    own = dtype == torch.float32 and len(shape) == 3 and solver in ("cg", "jacobi")
+    return ((0,) if own else ()) + ROW_CANDIDATES
+
+
+def _current(entry: Optional[dict]) -> Optional[dict]:
+    return entry if entry is not None and entry.get("engine") == ENGINE else None
 
 
 def _gpu_name(device) -> str:
@@ -118,9 +134,9 @@ def tune(shape, op_kind: str, solver: str, team: str = "grid", dtype=torch.float
     key = tune_key(_gpu_name(device), solver, op_kind, shape, dname, team)
     with _LOCK:
         cache = load_cache(path)
-        if not force and key in cache:
+        if not force and _current(cache.get(key)):
             return cache[key]
-    rows = rows or (ROW_CANDIDATES if team == "grid" else (8,))
+    rows = rows or row_candidates(shape, solver, dtype, team)
     nz = shape[2] if len(shape) >= 3 else 1
     planes = planes or tuple(p for p in PLANE_CANDIDATES if p == 0 or p < nz)
     trials = []
@@ -130,7 +146,8 @@ def tune(shape, op_kind: str, solver: str, team: str = "grid", dtype=torch.float
             trials.append({"tile_rows": r, "tile_planes": p, "ms_per_iter": ms})
     best = min(trials, key=lambda t: t["ms_per_iter"])
     entry = {"tile_rows": best["tile_rows"], "tile_planes": best["tile_planes"],
-             "ms_per_iter": best["ms_per_iter"], "trials": trials, "shape": list(shape)}
+             "ms_per_iter": best["ms_per_iter"], "trials": trials, "shape": list(shape),
+             "engine": ENGINE}
     with _LOCK:
         cache = load_cache(path)
         cache[key] = entry
@@ -143,7 +160,7 @@ def lookup(shape, op_kind: str, solver: str, team: str = "grid", dtype=torch.flo
     """The cached entry for this configuration, or None."""
     dname = "f64" if dtype == torch.float64 else "f32"
     key = tune_key(_gpu_name(device), solver, op_kind, shape, dname, team)
-    return load_cache(path).get(key)
+    return _current(load_cache(path).get(key))
 
 
 SMALL_BUCKET = 64
