@@ -492,6 +492,11 @@ const char *hs_last_error(void);
  * diffusion CG with TMA-staged planes (hs_opts.staging = 1), else 0. */
 int hs_last_staging(void);
 
+/* 1 if the last hs_jacobi or hs_cg solve (or inner CG of hs_solve_mixed) of the
+ * calling thread ran with four nodes per lane (FP32 on 3-D grids, see
+ * hs_opts.tile_rows), else 0. */
+int hs_last_quads(void);
+
 /* Library version string. */
 const char *hs_version(void);
 

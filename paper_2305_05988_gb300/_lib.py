@@ -115,6 +115,7 @@ SIGNATURES = {
     "hs_diag_fp64_rate": (_i, [_vp, ctypes.POINTER(_d)]),
     "hs_last_error": (ctypes.c_char_p, []),
     "hs_last_staging": (_i, []),
+    "hs_last_quads": (_i, []),
     "hs_version": (ctypes.c_char_p, []),
 }
 

@@ -16,6 +16,8 @@ static thread_local char g_err[512] = "no error";
 static thread_local int g_last_staging = 0;
 
 void set_last_staging(int v) { g_last_staging = v; }
+static thread_local int g_last_quads = 0;
+void set_last_quads(int v) { g_last_quads = v; }
 
 void set_error(const char* fmt, ...) {
   va_list ap;
@@ -249,6 +251,7 @@ extern "C" {
 const char* hs_last_error(void) { return g_err; }
 const char* hs_version(void) { return "hsolve 0.1 (sm_103a)"; }
 int hs_last_staging(void) { return g_last_staging; }
+int hs_last_quads(void) { return g_last_quads; }
 
 hs_status hs_diag_wait_timeout(int kind, double timeout_s, void* stream) {
   if (kind < 0 || kind > 3) {

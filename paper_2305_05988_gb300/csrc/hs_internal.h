@@ -240,5 +240,8 @@ hs_status cg32v_core(const hs_op* A, const float* k32, const float* b, float* x,
 // Thread-local record of whether the last solve staged its stencil planes
 // with TMA (hs_last_staging).
 void set_last_staging(int v);
+// Thread-local record of whether the last Jacobi or CG kernel had four nodes
+// per lane (hs_last_quads).
+void set_last_quads(int v);
 
 }  // namespace hs

@@ -168,12 +168,12 @@ struct JacobiSink {
   }
 };
 
-// Register caps of the neighbour-sum engine's kernels (A/B at 256^3; CG and
-// BiCGStab in 3-D):
-// Jacobi 64 (107 us per sweep; 48: 125, 56: 111, 80: 110; 2-D too: upwind
-// 2048^2 60.6 us without a cap, 53; with a residual 3000 x 2000 147 and 96), CG 80 (241 us per
-// iteration; 56: 278, 64: 258, 72: 250, 96: 283), BiCGStab 80 (527; 64: 642,
-// 96: 570, 128: 552).
+// Register caps of the neighbour-sum engine's kernels (A/B at 256^3 in long
+// solves, when the engine was built; CG and BiCGStab: 3-D): Jacobi 64 (107 us
+// per sweep; 48: 125, 56: 111, 80: 110; 2-D too: upwind 2048^2 60.6 us without a
+// cap, 53 with it; with a residual 3000 x 2000 147 and 96), CG 80 (241 us per
+// iteration; 56: 278, 64: 258, 72: 250, 96: 283), BiCGStab 80 (527; 64: 642, 96:
+// 570, 128: 552).
 #ifndef HS_JAC_ISO_MAXNREG
 #define HS_JAC_ISO_MAXNREG 64
 #endif
@@ -306,7 +306,7 @@ constexpr int cg_maxnreg() {
   if (fx_op(OPK) && NDIM == 3) return HS_CG_ISO_MAXNREG;
   if (sizeof(T) == 4) return (HS_CG32_MAXNREG > 0 && OPK == OP_VARK) ? HS_CG32_MAXNREG : 255;
   if (OPK == OP_VARK) return HS_CGV64_MAXNREG > 0 ? HS_CGV64_MAXNREG : 255;
-  if (OPK == OP_BOX27) return 72;   // 128 x 128 x 512: 278.8 us per iteration (64: 283.4, 80: 278.9)
+  if (OPK == OP_BOX27) return 72;   // 128 x 128 x 512, 10 iterations: 308 us each (64: 314)
   return HS_CG_MAXNREG > 0 ? HS_CG_MAXNREG : 255;
 }
 template <typename T, int OPK, int NDIM>
@@ -919,6 +919,7 @@ hs_status run_jacobi(const SolveArgs& sa, hs_result* res, double* hist) {
                    : launch(k_jacobi<T, OPK, NDIM, false, CX_QUAD>, 256, QR, QTW / BX, smem);
       }
     }
+    set_last_quads(quad ? 1 : 0);
     if (!quad) {
       const int by = rows_for(g, sa.o);
       constexpr int cx = cx_jac<T, OPK>();
@@ -964,11 +965,13 @@ static hs_status cg_core(const hs_op* A, const Coef<T>& cf, double sigma, const 
   };
   if constexpr (std::is_same<T, float>::value && NDIM == 3 && OPK != OP_BOX27) {
     if (quad_applies(a.g, o)) {
+      set_last_quads(1);
       constexpr size_t smem = std::max(quad_bytes<LoadSrc<T, true>, ResidualSink<T, OPK, NDIM>>(),
                                        quad_bytes<PUpdateSrc<T>, ApDotSink<T, OPK, NDIM, false>>());
       return launch(k_cg<T, OPK, NDIM, CX_QUAD>, 256, QR, QTW / BX, smem);
     }
   }
+  set_last_quads(0);
   const int by = rows_for(a.g, o);
   constexpr int cx = cx_cg<T, OPK>();
   return launch(k_cg<T, OPK, NDIM, cx>, 32 * by, by, cx, slab_bytes<T, OPK, NDIM>(by, cx, 2, 1));
@@ -1212,7 +1215,8 @@ hs_status run_mixed(const SolveArgs& sa, hs_result* res, double* hist) {
   hs_status s;
   // FP32 inner CG on a 3-D diffusion operator with staging 1: the TMA-staged
   // kernel with the face coefficients formed from k (L.D32 then holds k in
-  // FP32); otherwise the register-prefetch engine on stored FP32 coefficients
+  // FP32); otherwise on stored FP32 coefficients, four nodes per lane where
+  // quad_applies, else the register-prefetch engine
   const bool tma = sa.o.inner_solver != HS_SOLVER_BICGSTAB && sa.o.staging == 1 && cg32v_eligible(A, sa.o);
   if (!tma && sa.o.staging == 1) {
     set_error("TMA staging requested but this problem does not allow it (3-D diffusion, inner CG, n_x a "
