@@ -69,7 +69,7 @@ FLOPS = {"spmv": 3.0, "jacobi": 2.0, "gauss_seidel": 9.0, "cg": 12.0, "bicgstab"
 # subtracted).  Traffic grows with unknowns x iterations (each pass streams
 # every vector), so a launch of the step moves this figure x N x iterations.
 # Re-measure whenever the kernel changes.
-TRAFFIC_B_PER_UNIT = {"cg": 74.8, "bicgstab": 138.8, "jacobi": 25.2}
+TRAFFIC_B_PER_UNIT = {"cg": 74.1, "bicgstab": 135.8, "jacobi": 25.4}
 # FP64 pipe: 2 FMA lanes per SM per clock (ncu: sm__sass_thread_inst_executed_op_dfma_pred_on
 # peak_sustained = 2 per SM per cycle) x 2 flops x 152 SMs.
 FP64_FLOPS_PER_CLK = 2 * 2 * 152

@@ -131,9 +131,9 @@ typedef struct {
                                them).                                          */
     int staging;            /* FP32 CG on a 3-D diffusion operator (hs_cg with
                                HS_F32, and the inner CG of hs_solve_mixed):
-                               0 (default) the register-prefetch tile engine
-                               on stored FP32 coefficient arrays (16 B of
-                               operator data per node, the fastest measured);
+                               0 (default) the tile engines on stored FP32
+                               coefficient arrays (16 B of operator data per
+                               node, the fastest measured; see tile_rows);
                                1 the stencil planes staged in shared memory by
                                TMA and the face coefficients formed from k
                                (4 B per node; 3-D, n_x a multiple of 4,

@@ -12,9 +12,11 @@
 // planes early and ends S planes late for the same reason as the rings.
 //
 // Per node and sweep this trades 24 (FP64) / 12 (FP32) bytes of HBM traffic
-// for 24 / L (12 / L) bytes plus the recomputed rings.  On GB300 FP64 Jacobi is
-// bound by the FP64 pipe, not by HBM, so blocking pays for FP32 sweeps (memory
-// bound) and costs FP64 ones the ring recomputation; both are measured.
+// for 24 / L (12 / L) bytes plus the recomputed rings.  On GB300 neither single
+// sweep is bound by HBM alone (FP64: instruction issue; FP32: four nodes per
+// lane, three quarters of the traffic's rate), so the rings cost more than the
+// bytes saved: 256^3, us per sweep at 1 / 2 / 3 / 4 sweeps per pass, FP64 112 / 229
+// / 287 / 316, FP32 39.5 / 110 / 98 / 147.
 //
 // Every node runs the same Jacobi-form arithmetic as k_jacobi (jacobi_apply,
 // same operand order, the same neighbour sum), so the iterates are

@@ -27,6 +27,7 @@ constexpr int BX = 32;
 #define HS_FX_NS 4
 #endif
 constexpr int FX_NS = HS_FX_NS;   // ring stages of the neighbour-sum engine
+static_assert(FX_NS >= 2 && (FX_NS & (FX_NS - 1)) == 0, "steps map to stages by masking");
 
 struct Tiling {
   int by;        // rows per tile (3..16), blockDim.x = 32 * by
@@ -427,13 +428,14 @@ __device__ __forceinline__ void zmarch_box(const Geom& g, const Tiling& tl, int 
 // L1; a value rewritten by another block was ordered by the grid barrier's
 // acquire, which also drops stale L1 lines.
 //
-// 256^3 FP64, before (zmarch_item, additions on the FP64 pipe) and now: Jacobi
-// 220 -> 114 us per sweep (59 us of traffic), CG 411 -> 245 us per iteration,
-// SpMV 256 -> 122 us, residual 327 -> 181 us; weighted (250 x 187 x 141):
-// Jacobi 99 -> 64, CG 191 -> 129, BiCGStab 392 -> 284; upwind at 256^3: Jacobi
-// 221 -> 167, BiCGStab 858 -> 603.  Tried and slower: operands
-// prefetched in registers as in zmarch_item (Jacobi 135, CG 289), one plane
-// ahead only (Jacobi 173), the loop unrolled six times so that no register
+// 256^3 FP64, before (zmarch_item, additions on the FP64 pipe) and now, short
+// calls (20 sweeps or iterations, BiCGStab 10) on a flushed L2: Jacobi 224 -> 115
+// us per sweep (59 us of traffic), CG 434 -> 264 us per iteration, SpMV 242 ->
+// 109 us, residual 308 -> 145 us; weighted (250 x 187 x 141): Jacobi 101 -> 71,
+// CG 203 -> 135, BiCGStab (upwind) 408 -> 298; upwind at 256^3: Jacobi 224 -> 174, BiCGStab 892
+// -> 631.  Tried and slower, when Jacobi took 114 and CG 245 in long solves:
+// operands prefetched in registers as in zmarch_item (Jacobi 135, CG 289), one
+// plane ahead only (Jacobi 173), the loop unrolled six times so that no register
 // moves (CG 366: the code leaves the instruction cache), two rows per lane
 // (Jacobi 149).
 //
