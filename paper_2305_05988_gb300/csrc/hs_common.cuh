@@ -178,13 +178,13 @@ __device__ __forceinline__ int ld_acquire_int(const int* p) {
 // before each solve).
 struct Ctrl {
   unsigned count;        // arrivals at the team's barriers (only grows; LastTeam: at this one)
-  unsigned gen;          // barrier generation (LastTeam)
+  unsigned gen;          // barrier generation (LastTeam, BiTeam)
   int status;            // DevStatus
   int iters;             // iterations completed
   int restarts;          // BiCGStab restarts
   int pad0;
   unsigned long long timeout_ns;
-  double scal[16];       // reduced scalars of the last barrier (LastTeam)
+  double scal[16];       // reduced scalars of the last barrier (LastTeam, BiTeam)
   double rel_res;        // last relative residual
   double aux[7];
 };

@@ -1,6 +1,6 @@
 // hs_diag.cu -- hs_diag_fp64_rate: the FP64 fused multiply-add rate this GPU
 // sustains, measured with independent dependency chains in every thread.  FP64
-// CG, BiCGStab and Gauss-Seidel keep that pipe 70 to 76 % busy (a 7-point
+// CG, BiCGStab and Gauss-Seidel keep that pipe 70 to 75 % busy (a 7-point
 // stencil of FP64 additions alone, about 6 instructions per node, takes longer
 // than its 24 bytes of traffic at HBM speed on this part), so the benchmark
 // divides their flop rates by this measurement.
